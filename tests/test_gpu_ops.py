@@ -97,6 +97,28 @@ def test_vocab_signals(V, d):
         assert int(tok.item()) == c["argmax"]
 
 
+@pytest.mark.parametrize("n", [31, 2431, 2432, 4864, 9728, 19456, 38912, 77824])
+def test_select_tau_slices(n):
+    """Each number of lanes a candidate is shared by, at and past its largest
+    n, against the counts of every candidate taken from a sort."""
+    import torch
+
+    from paper_2609_14144_gb300 import select_tau
+
+    rng = np.random.default_rng(n)
+    conf = (np.floor(rng.random(n) * 3 * n) / (3 * n)).astype(np.float32)
+    member = (rng.random(n) < 0.4 + 0.6 * conf).astype(np.int32)
+    cs, good = np.sort(conf), None
+    order = np.argsort(conf, kind="stable")
+    good = np.concatenate([np.cumsum(member[order][::-1])[::-1], [0]])
+    cands = np.concatenate([[-np.inf], np.unique(cs)])
+    at = np.searchsorted(cs, cands, side="right")
+    for target in (0.5, 0.9):
+        ok = (n - at > 0) & (good[at] >= np.float64(np.float32(target)) * (n - at))
+        want = cands[ok].min() if ok.any() else np.inf
+        assert select_tau(_dev(conf), _dev(member), target).item() == np.float32(want)
+
+
 def test_vocab_signals_tie_and_uniform():
     import torch
 
