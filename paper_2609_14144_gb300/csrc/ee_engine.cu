@@ -1549,7 +1549,12 @@ int vocab_standalone(const float* x, const uint16_t* gain, const uint16_t* U, in
     v.out_p = out_p;
     v.out_sig = out_sig;
     EE_CK(cudaMemsetAsync(v.ticket, 0, 4, s));
-    EE_CK(launch_vocab(v, std::min(nsm, kMaxVocabCtas), false, s));
+    // the ring wants 16-byte rows on 16-byte boundaries (the d_model % 8 that
+    // ee_vocab_scratch_bytes checks) and the row's columns in registers
+    if (d_model <= kVocabRowsMaxD)
+        EE_CK(launch_vocab_rows(v, std::min(nsm, kMaxVocabCtas), s));
+    else
+        EE_CK(launch_vocab(v, std::min(nsm, kMaxVocabCtas), false, s));
     return EE_OK;
 }
 }  // namespace

@@ -224,6 +224,15 @@ __device__ __forceinline__ float warp_max(float v) {
     for (int o = 16; o; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
 }
+// a * b + c on two packed floats (round to nearest, as fmaf on each).
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;"
+        : "=l"(reinterpret_cast<unsigned long long&>(d))
+        : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)),
+          "l"(reinterpret_cast<const unsigned long long&>(c)));
+    return d;
+}
 __device__ __forceinline__ float dot8s(const uint4 w, uint32_t xa) {
     const float4 a = lds128f(xa);
     const float4 b = lds128f(xa + 16);
@@ -1531,6 +1540,127 @@ __global__ void __launch_bounds__(kSegThreads, 1) k_vocab_ring(VocabArgs v, int 
     vocab_finish(v, st, nucleus, kCW, [] { csync(); });
 }
 
+// The vocabulary pass over a caller's row-major U [V, d] (standalone ops).
+// CTA b streams its contiguous rows through the ring, kVrRows rows (at most
+// kSegChunk bytes) a stage; a warp takes whole rows of a stage, kVrBatch at a
+// time, lane = 16-byte column chunks lane, lane + 32, ... (one conflict-free
+// 512-byte load per step), with the normalised input's columns of those chunks
+// kept in registers for the whole pass (KC of them: d <= 256 KC).  A row's
+// sum ends on the lane of its turn, so that the softmax statistics of 32 rows
+// are updated together.  HBM bounds it (2 V d bytes); a streaming launch of
+// one 512-thread CTA per SM with the loads of one row in flight per warp took
+// 113.1 us a call for 151936 x 1536 (4.1 TB/s), the ring 89.4 us (5.2 TB/s).
+constexpr int kVrBatch = 2;  // rows a warp reduces together
+constexpr int vr_rows(int d) {  // rows a stage: as many as fit, in whole turns of the warps
+    return kSegChunk / (2 * d) >= kCW * kVrBatch ? kSegChunk / (2 * d) / (kCW * kVrBatch) * (kCW * kVrBatch)
+                                                 : kSegChunk / (2 * d);
+}
+template <int KC>
+__global__ void __launch_bounds__(kSegThreads, 1) k_vocab_rows(VocabArgs v, int stages, int rows) {
+    extern __shared__ __align__(128) uint8_t vr_smem[];
+    __shared__ int err_local;
+    __shared__ float nss[kCW];
+    Smem s{};
+    s.ring = vr_smem;
+    s.full = reinterpret_cast<uint64_t*>(vr_smem + (size_t)stages * kSegChunk);
+    s.empty = s.full + stages;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        err_local = 0;
+        for (int i = 0; i < stages; ++i) {
+            mb_init(&s.full[i], 1);
+            mb_init(&s.empty[i], kCW);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    const Waits wt{&err_local, kSegStallCycles, kSegCheckCycles};
+    const int r0 = (int)((int64_t)v.V * blockIdx.x / gridDim.x), r1 = (int)((int64_t)v.V * (blockIdx.x + 1) / gridDim.x);
+    if (threadIdx.x >= kCT) {  // producer
+        if (threadIdx.x != kCT) return;
+        Producer pr(s, stages, stages, wt);
+        for (int r = r0; r < r1 && pr.ok; r += rows)
+            pr.push(v.U + (int64_t)r * v.d, (uint32_t)(min(rows, r1 - r) * v.d * 2), pr.pol_w);
+        pr.drain();
+        return;
+    }
+    Consumer cs(s, stages, wt);
+    // RMSNorm(x) * gain, this lane's columns
+    float ss = 0.f;
+    for (int i = threadIdx.x; i < v.d; i += kCT) ss = fmaf(v.x[i], v.x[i], ss);
+    ss = warp_sum(ss);
+    if (lane == 0) nss[w] = ss;
+    csync();
+    float tot = 0.f;
+#pragma unroll
+    for (int k = 0; k < kCW; ++k) tot += nss[k];
+    const float inv = 1.0f / sqrtf(tot / (float)v.d + v.eps);
+    const int Rc = v.d >> 3;
+    float2 x[KC][4];
+#pragma unroll
+    for (int k = 0; k < KC; ++k) {
+        const int c = lane + 32 * k;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int i = 8 * c + 2 * e;
+            x[k][e] = c < Rc ? make_float2(v.x[i] * inv * bf(v.gain[i]), v.x[i + 1] * inv * bf(v.gain[i + 1]))
+                             : make_float2(0.f, 0.f);
+        }
+    }
+    SoftStats st;
+    float mine = 0.f;
+    int mine_row = -1, turn = 0;  // the row sum this lane holds; rows since the last update
+    auto update = [&]() {
+        if (mine_row >= 0) {
+            if (v.logits) v.logits[mine_row] = mine;
+            st.add(mine, mine_row);
+        }
+        mine_row = -1;
+        turn = 0;
+    };
+    for (int rb = r0; rb < r1; rb += rows) {
+        const uint32_t base = saddr(cs.acquire()) + lane * 16;
+        const int nr = min(rows, r1 - rb);
+        if (cs.ok) {
+#pragma unroll 1
+            for (int r = w * kVrBatch; r < nr; r += kCW * kVrBatch) {
+                float2 acc[kVrBatch][2];
+#pragma unroll
+                for (int b = 0; b < kVrBatch; ++b) acc[b][0] = acc[b][1] = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int k = 0; k < KC; ++k) {
+                    if (lane + 32 * k < Rc) {
+#pragma unroll
+                        for (int b = 0; b < kVrBatch; ++b) {
+                            // (a row past the stage's rows reads the ring's next bytes: not used)
+                            const uint4 u = lds128(base + min(r + b, nr - 1) * v.d * 2 + k * 512);
+                            acc[b][0] = fma2(make_float2(bflo(u.x), bfhi(u.x)), x[k][0], acc[b][0]);
+                            acc[b][1] = fma2(make_float2(bflo(u.y), bfhi(u.y)), x[k][1], acc[b][1]);
+                            acc[b][0] = fma2(make_float2(bflo(u.z), bfhi(u.z)), x[k][2], acc[b][0]);
+                            acc[b][1] = fma2(make_float2(bflo(u.w), bfhi(u.w)), x[k][3], acc[b][1]);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int b = 0; b < kVrBatch; ++b) {
+                    const float t = warp_sum((acc[b][0].x + acc[b][0].y) + (acc[b][1].x + acc[b][1].y));
+                    if (r + b < nr) {
+                        if (lane == turn) {
+                            mine = t;
+                            mine_row = rb + r + b;
+                        }
+                        ++turn;
+                    }
+                }
+                if (turn > 32 - kVrBatch) update();
+            }
+        }
+        cs.release();
+    }
+    update();
+    vocab_finish(v, st, false, kCW, [] { csync(); });
+}
+
 }  // namespace
 
 bool vocab_ring_plan(int d, int n_sm, VocabRing& vr) {
@@ -1560,6 +1690,22 @@ cudaError_t launch_vocab_ring(const VocabArgs& v, const VocabRing& vr, bool pdl,
     cfg.attrs = at;
     cfg.numAttrs = pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, k_vocab_ring, v, vr.stages);
+}
+
+cudaError_t launch_vocab_rows(const VocabArgs& v, int n_sm, cudaStream_t s) {
+    if (v.d > kVocabRowsMaxD || v.d % 8 || v.mode != 0) return cudaErrorInvalidValue;
+    constexpr int stages = 6;
+    const size_t smem = stages * (size_t)(kSegChunk + 16);
+    auto go = [&](auto kern) -> cudaError_t {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        kern<<<n_sm, kSegThreads, smem, s>>>(v, stages, vr_rows(v.d));
+        return cudaGetLastError();
+    };
+    if (v.d <= 512) return go(k_vocab_rows<2>);
+    if (v.d <= 1024) return go(k_vocab_rows<4>);
+    if (v.d <= 1536) return go(k_vocab_rows<6>);
+    return go(k_vocab_rows<8>);
 }
 
 bool seg_plan(const DevModel& m, int n_sm, SegPlan& p) {

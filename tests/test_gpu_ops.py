@@ -74,6 +74,34 @@ def test_vocab_confidence(V, d):
         assert int(tok.item()) == c["argmax"]
 
 
+@pytest.mark.parametrize("V", [2, 151, 2433, 20011])
+@pytest.mark.parametrize("d", [256, 264, 512, 520, 1024, 1032, 1536, 1544, 2040, 2048, 2056])
+def test_vocab_rows_widths(V, d):
+    """Row widths at the edges of the columns a lane keeps in registers, ragged
+    last column chunks, fewer rows than CTAs, partly filled stages, and the
+    first width past the ring's.  Logits within the fp32 summation bound, the
+    token the highest logit's lowest index."""
+    import torch
+
+    from paper_2609_14144_gb300 import vocab_signals
+
+    g = torch.Generator(device="cuda").manual_seed(V * 7 + d)
+    x = torch.randn(d, generator=g, device="cuda")
+    gain = torch.randn(d, generator=g, device="cuda").to(torch.bfloat16)
+    U = torch.randn(V, d, generator=g, device="cuda").to(torch.bfloat16)
+    logits = torch.full((V,), float("nan"), device="cuda")
+    tok, sig = vocab_signals(x, gain, U, 1e-6, logits=logits)
+    z = x.double() / torch.sqrt((x.double() ** 2).mean() + 1e-6) * gain.double()
+    ref = U.double() @ z
+    bound = (U.double().abs() @ z.abs()) * 2.0 ** -24 * (d / 64 + 8)
+    assert ((logits.double() - ref).abs() <= bound).all()
+    assert tok.item() == logits.argmax().item()
+    p = torch.softmax(logits.double(), 0)
+    top = torch.topk(p, 2).values
+    want = torch.stack([top[0], top[0] - top[1], (p * torch.log_softmax(logits.double(), 0)).sum()])
+    assert (sig.double() - want).abs().max().item() <= 1e-5 * max(1.0, want.abs().max().item())
+
+
 @pytest.mark.parametrize("V,d", [(4096, 256), (151936, 1536), (1000, 2048)])
 def test_vocab_signals(V, d):
     """Section 10's three signals from one pass, against the oracle's
