@@ -367,7 +367,7 @@ int ee_attention_decode(const float* q, const uint16_t* k_pages, const uint16_t*
  *   process exits.  Shapes needing more (n_heads * (head_dim + 2) above about
  *   4096) are rejected with EE_EINVAL and a message.
  *   The area is shared by every call and keeps the previous call's contents;
- *   each call clears the part that must start at zero.  Calls whose work
+ *   nothing in it has to be cleared.  Calls whose work
  *   overlaps on the GPU (other streams, other threads) race on the area:
  *   order them on one stream.
  *   Every call looks up the area's device address on the current device

@@ -57,7 +57,7 @@ int64_t align_elems(int64_t x) { return (x + 127) / 128 * 128; }  // 256 bytes o
 struct Layout {
     size_t ctl, rope, layers, embed, lm_head, g_final, ro_w[kMaxReadouts], ro_b[kMaxReadouts];
     size_t kpool, vpool, page_table, kv_src, h_exit, exit_at, repass_pos, h, q, o, a, y, hk, logits_ro, logits_final;
-    size_t gemv_part, gemv_ticket, attn_part, attn_ticket, vocab_part, vocab_ticket;
+    size_t gemv_part, gemv_ticket, vocab_part, vocab_ticket;
     size_t seg_dpart, seg_opart, seg_q, seg_kvn, seg_a, seg_attn, seg_sync, seg_end;
     size_t rows_H, rows_x3, rows_Q, rows_part, rows_pos;
     size_t prompt, sched, out_tok, out_exit, out_conf, out_conf_all, out_member, out_mass, tau_scratch, total;
@@ -148,8 +148,6 @@ Layout make_layout(const ee_model_config& c) {
     l.logits_final = take(4 * (size_t)V);
     l.gemv_part = take(4 * (size_t)(kMaxGemvCtas + L) * 2 * kTileRows);
     l.gemv_ticket = take(4 * (size_t)l.gemv_ticket_stride * L);
-    l.attn_part = take(4 * (size_t)A * kAttnMaxSplits * (D + 2));
-    l.attn_ticket = take(4 * (size_t)KH);
     l.vocab_part = take(4 * (size_t)kMaxVocabCtas * 8);
     l.vocab_ticket = take(4);
     // persistent layer kernel: down-projection partials, mid residual, counters
@@ -296,8 +294,6 @@ AttnArgs attn_args(const ee_ctx* c, int j) {
     a.KH = m.KH;
     a.page_size = m.page_size;
     a.out = m.o;
-    a.part = m.attn_part;
-    a.ticket = m.attn_ticket;
     return a;
 }
 
@@ -854,8 +850,6 @@ int ee_create(const ee_model_config* cfg, void* d_workspace, size_t workspace_by
     m.gemv_part = (float*)(w + l.gemv_part);
     m.gemv_ticket = (unsigned*)(w + l.gemv_ticket);
     m.gemv_ticket_stride = l.gemv_ticket_stride;
-    m.attn_part = (float*)(w + l.attn_part);
-    m.attn_ticket = (int*)(w + l.attn_ticket);
     m.vocab_part = (float*)(w + l.vocab_part);
     m.vocab_ticket = (int*)(w + l.vocab_ticket);
     m.ctl = (Ctl*)(w + l.ctl);
@@ -910,7 +904,6 @@ int ee_create(const ee_model_config* cfg, void* d_workspace, size_t workspace_by
         return bail(fail(EE_ECUDA, "page table upload failed"));
     // zero the arrival counters (kernels return them to zero after use)
     if (cudaMemset(w + l.gemv_ticket, 0, 4 * (size_t)l.gemv_ticket_stride * m.L) != cudaSuccess ||
-        cudaMemset(w + l.attn_ticket, 0, 4 * (size_t)m.KH) != cudaSuccess ||
         cudaMemset(w + l.vocab_ticket, 0, 4) != cudaSuccess)
         return bail(fail(EE_ECUDA, "memset failed"));
     *out = c;
@@ -1493,7 +1486,6 @@ int ee_attention_decode(const float* q, const uint16_t* k_pages, const uint16_t*
     if (page_size <= 0) return fail(EE_EINVAL, "bad page size");
     if (scratch_bytes < need) return fail(EE_ENOMEM, "scratch too small");
     cudaStream_t s = (cudaStream_t)stream;
-    char* sc = (char*)scratch;
     AttnArgs a{};
     a.q = q;
     a.kp = k_pages;
@@ -1505,10 +1497,8 @@ int ee_attention_decode(const float* q, const uint16_t* k_pages, const uint16_t*
     a.KH = n_kv_heads;
     a.page_size = page_size;
     a.out = out;
-    a.part = (float*)sc;
-    a.ticket = (int*)(sc + align_up(4 * (size_t)n_heads * kAttnMaxSplits * (head_dim + 2)));
-    EE_CK(cudaMemsetAsync(a.ticket, 0, 4 * (size_t)n_kv_heads, s));
-    EE_CK(launch_attention(a, head_dim, false, s));
+    a.part = (float*)scratch;
+    EE_CK(launch_attention(a, head_dim, s));
     return EE_OK;
 }
 

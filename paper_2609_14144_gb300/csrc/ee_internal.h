@@ -12,7 +12,6 @@ namespace ee {
 constexpr int kMaxReadouts = EE_MAX_READOUTS;
 constexpr int kGemvThreads = 512;   // 16 warps per CTA in the streaming GEMVs
 constexpr int kAttnThreads = 256;   // 8 warps per CTA in split-K attention
-constexpr int kAttnMinRows = 32;    // positions per attention split (at least)
 constexpr int kAttnMaxSplits = 128; // splits per key-value head (at most)
 
 // Bits of the device error word.
@@ -98,8 +97,6 @@ struct DevModel {
     float* gemv_part;             // cross-CTA tile partials: [CTA slot][2][32]
     unsigned* gemv_ticket;        // per-tile arrival counters
     int64_t gemv_ticket_stride;   // counters per fill layer in gemv_ticket
-    float* attn_part;             // [A][kAttnMaxSplits][D + 2]
-    int* attn_ticket;             // [KH]
     float* vocab_part;            // [grid][8]
     int* vocab_ticket;            // [1]
     Ctl* ctl;
@@ -115,8 +112,7 @@ struct AttnArgs {
     int T;
     int A, KH, page_size;
     float* out;
-    float* part;
-    int* ticket;
+    float* part;              // standalone op: [A][kAttnMaxSplits][D + 2]
 };
 
 // Arguments of the vocabulary pass (readout / LM head / standalone).
@@ -161,7 +157,7 @@ struct CtlInputs {
 // `pdl` adds the programmatic-stream-serialisation attribute.
 // `whole`: one CTA per tile, the tile staged in shared memory before the wait.
 cudaError_t launch_qkv(const DevModel& m, int layer, int first, int grid, bool whole, bool pdl, cudaStream_t s);
-cudaError_t launch_attention(const AttnArgs& a, int head_dim, bool pdl, cudaStream_t s);
+cudaError_t launch_attention(const AttnArgs& a, int head_dim, cudaStream_t s);
 // The engine's attention: one thread-block cluster of `cluster` CTAs per kv head.
 cudaError_t launch_attention_cluster(const AttnArgs& a, int head_dim, int cluster, bool pdl, cudaStream_t s);
 // Largest cluster size (16 or 8) the attention kernel can be resident with.

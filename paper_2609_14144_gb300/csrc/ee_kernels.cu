@@ -973,158 +973,236 @@ __global__ void __launch_bounds__(kGemvThreads, 2) k_vocab_rowmajor(VocabArgs v)
     vocab_finish(v, st, false, (int)(blockDim.x >> 5), [] { __syncthreads(); });
 }
 
-// Split-K decode attention over the paged cache.  Grid (splits, KH): CTA
-// (s, g) covers a contiguous run of positions for the A/K query heads of
-// key-value head g with a per-lane online softmax; the last CTA of head g
-// merges the splits and writes o = softmax(q K^T / sqrt(D)) V (fp32).
-template <int D>
-__global__ void __launch_bounds__(kAttnThreads) k_attention(AttnArgs a) {
-    constexpr int LPR = D / 8;  // lanes per position (8 dims each)
-    constexpr int RPW = 32 / LPR;
+// Split-K decode attention over the paged cache (the standalone op), two
+// launches.  k_attn_split: grid (S, KH), CTA (s, g) covers positions
+// [s * chunk, (s + 1) * chunk) for the G = A / K query heads of key-value head
+// g, its eight warps taking tiles of 16 positions in turn.  A tile's keys and
+// values go straight to registers, all of their loads issued together: at
+// these sizes (16 MB spread over the GPU leaves 16 to 32 positions a warp) the
+// op is a chain of latencies, page table -> rows -> scores -> output, so every
+// load of a tile is in flight at once and nothing is staged.  Scores: lanes
+// (g8, t4) hold 8-dimension chunks t4 of keys g8 and g8 + 8, each chunk of the
+// query is read once for both.  P V: lane = D / 32 dimensions, a position's
+// probabilities of all heads are one or two 16-byte loads.  k_attn_merge
+// combines the splits, one CTA per (head, 32 dimensions).
+// A call at 12/2 heads of 128 and 16411 positions takes 18.4 us (of which the
+// host's two launches 18), 96.6 us for a per-lane online softmax over every
+// position with the merge in the last CTA of a head (two exponentials per
+// position and head, and a serial merge of 128 splits).
+constexpr int kAttnTile = 16;  // positions per warp and tile
+template <int D, int G>
+__global__ void __launch_bounds__(kAttnThreads, 2) k_attn_split(AttnArgs a, int chunk) {
+    constexpr int PR = D / 32;   // 16-byte chunks a lane holds of one key; dimensions it holds of the output
+    constexpr int GP = (G + 3) & ~3;
     constexpr int NW = kAttnThreads / 32;
-    constexpr int GMAX = 8;
-    __shared__ __align__(16) float qs[GMAX * D];
-    __shared__ float wm[NW][GMAX], wl[NW][GMAX];
-    __shared__ __align__(16) float wacc[NW][GMAX][D];
-    __shared__ int is_last;
-    pdl_wait();
+    __shared__ __align__(16) float qs[G * D];
+    __shared__ __align__(16) float ps[NW][kAttnTile][GP];
+    __shared__ float wm[NW][8], wl[NW][8], wgt[NW][8];
+    __shared__ __align__(16) float wacc[NW][G][D];
     pdl_launch_dependents();
-    const int T = a.ctl ? a.ctl->pos + 1 : a.T;
-    const int G = a.A / a.KH;
-    int S = (T + kAttnMinRows - 1) / kAttnMinRows;
-    if (S > (int)gridDim.x) S = gridDim.x;
-    const int chunk = (T + S - 1) / S;
     const int s = blockIdx.x, g = blockIdx.y;
-    if (s >= S) return;
-    const int t0 = s * chunk, t1 = min(T, t0 + chunk);
-    const float scale = 1.0f / sqrtf((float)D);
-    for (int i = threadIdx.x; i < G * D; i += blockDim.x) qs[i] = a.q[(int64_t)g * G * D + i] * scale;
-    __syncthreads();
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int grp = lane / LPR, e0 = (lane % LPR) * 8;
-    float mx[GMAX], ls[GMAX], acc[GMAX][8];
-#pragma unroll
-    for (int h = 0; h < GMAX; ++h) {
-        mx[h] = -CUDART_INF_F;
-        ls[h] = 0.f;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) acc[h][e] = 0.f;
-    }
+    const int t0 = s * chunk, t1 = min(a.T, t0 + chunk);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g8 = lane >> 2, t4 = lane & 3;
     const int P = a.page_size;
-    for (int tt = t0 + warp * RPW; tt < t1; tt += NW * RPW) {
-        const int t = tt + grp;
-        const bool valid = t < t1;
-        float kf[8], vf[8];
-        if (valid) {
-            const int page = a.page_table[t / P];
-            const int64_t off = (((int64_t)page * a.KH + g) * P + (t % P)) * D + e0;
-            const uint4 kw = *reinterpret_cast<const uint4*>(a.kp + off);
-            const uint4 vw = *reinterpret_cast<const uint4*>(a.vp + off);
-            kf[0] = bf_lo(kw.x); kf[1] = bf_hi(kw.x); kf[2] = bf_lo(kw.y); kf[3] = bf_hi(kw.y);
-            kf[4] = bf_lo(kw.z); kf[5] = bf_hi(kw.z); kf[6] = bf_lo(kw.w); kf[7] = bf_hi(kw.w);
-            vf[0] = bf_lo(vw.x); vf[1] = bf_hi(vw.x); vf[2] = bf_lo(vw.y); vf[3] = bf_hi(vw.y);
-            vf[4] = bf_lo(vw.z); vf[5] = bf_hi(vw.z); vf[6] = bf_lo(vw.w); vf[7] = bf_hi(vw.w);
-        } else {
+    const float scale = 1.0f / sqrtf((float)D);
+    for (int i = threadIdx.x; i < G * D; i += kAttnThreads) qs[i] = a.q[(int64_t)g * G * D + i] * scale;
+
+    float mx[G], acc[G][PR], ls[2] = {0.f, 0.f};  // ls: heads t4 and t4 + 4, keys g8 and g8 + 8 of every tile
 #pragma unroll
-            for (int e = 0; e < 8; ++e) kf[e] = vf[e] = 0.f;
+    for (int h = 0; h < G; ++h) {
+        mx[h] = -CUDART_INF_F;
+#pragma unroll
+        for (int e = 0; e < PR; ++e) acc[h][e] = 0.f;
+    }
+    bool synced = false;
+    for (int tt = t0 + warp * kAttnTile; tt < t1; tt += NW * kAttnTile) {
+        // lane l < 16: element offset of position tt + l's row
+        int64_t off = 0;
+        if (lane < kAttnTile && tt + lane < t1) {
+            const int t = tt + lane, page = t / P;
+            off = (((int64_t)a.page_table[page] * a.KH + g) * P + (t - page * P)) * D;
         }
+        uint4 kw[2][PR];
 #pragma unroll
-        for (int h = 0; h < GMAX; ++h) {
-            if (h >= G) break;
-            float d = 0.f;
+        for (int u = 0; u < 2; ++u) {
+            const int64_t o = __shfl_sync(0xffffffffu, off, g8 + 8 * u);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) d = fmaf(kf[e], qs[h * D + e0 + e], d);
+            for (int r = 0; r < PR; ++r)
+                kw[u][r] = tt + g8 + 8 * u < t1 ? __ldg(reinterpret_cast<const uint4*>(a.kp + o + r * 32 + t4 * 8))
+                                                : make_uint4(0u, 0u, 0u, 0u);
+        }
+        uint2 vw[kAttnTile];
 #pragma unroll
-            for (int o = LPR / 2; o; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-            if (valid) {
-                const float mn = fmaxf(mx[h], d);
-                const float corr = expf(mx[h] - mn);
-                const float p = expf(d - mn);
-                ls[h] = ls[h] * corr + p;
+        for (int r = 0; r < kAttnTile; ++r) {
+            const int64_t o = __shfl_sync(0xffffffffu, off, r);
+            vw[r] = make_uint2(0u, 0u);
+            if (tt + r < t1) {
+                if (PR == 4)
+                    vw[r] = __ldg(reinterpret_cast<const uint2*>(a.vp + o) + lane);
+                else
+                    vw[r].x = __ldg(reinterpret_cast<const uint32_t*>(a.vp + o) + lane);
+            }
+        }
+        if (!synced) {  // the queries (their loads overlap the first tile's)
+            __syncthreads();
+            synced = true;
+        }
+        float sc[2][G];
 #pragma unroll
-                for (int e = 0; e < 8; ++e) acc[h][e] = fmaf(p, vf[e], acc[h][e] * corr);
-                mx[h] = mn;
+        for (int h = 0; h < G; ++h) sc[0][h] = sc[1][h] = 0.f;
+#pragma unroll
+        for (int r = 0; r < PR; ++r) {
+            float k0[8], k1[8];
+            const uint32_t w0[4] = {kw[0][r].x, kw[0][r].y, kw[0][r].z, kw[0][r].w};
+            const uint32_t w1[4] = {kw[1][r].x, kw[1][r].y, kw[1][r].z, kw[1][r].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                k0[2 * e] = bf_lo(w0[e]), k0[2 * e + 1] = bf_hi(w0[e]);
+                k1[2 * e] = bf_lo(w1[e]), k1[2 * e + 1] = bf_hi(w1[e]);
+            }
+#pragma unroll
+            for (int h = 0; h < G; ++h) {
+                const float4 qa = *reinterpret_cast<const float4*>(qs + h * D + r * 32 + t4 * 8);
+                const float4 qb = *reinterpret_cast<const float4*>(qs + h * D + r * 32 + t4 * 8 + 4);
+                const float q8[8] = {qa.x, qa.y, qa.z, qa.w, qb.x, qb.y, qb.z, qb.w};
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    sc[0][h] = fmaf(k0[e], q8[e], sc[0][h]);
+                    sc[1][h] = fmaf(k1[e], q8[e], sc[1][h]);
+                }
+            }
+        }
+        const bool ok0 = tt + g8 < t1, ok1 = tt + g8 + 8 < t1;
+        const bool first = tt < t0 + NW * kAttnTile;
+        __syncwarp();  // the previous tile's probabilities are read
+#pragma unroll
+        for (int h = 0; h < G; ++h) {
+            float s0 = sc[0][h], s1 = sc[1][h];
+            s0 += __shfl_xor_sync(0xffffffffu, s0, 1);
+            s1 += __shfl_xor_sync(0xffffffffu, s1, 1);
+            s0 += __shfl_xor_sync(0xffffffffu, s0, 2);
+            s1 += __shfl_xor_sync(0xffffffffu, s1, 2);
+            float m = fmaxf(ok0 ? s0 : -CUDART_INF_F, ok1 ? s1 : -CUDART_INF_F);
+#pragma unroll
+            for (int o = 4; o < 32; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+            m = fmaxf(m, mx[h]);
+            if (!first) {
+                const float c = expf(mx[h] - m);
+#pragma unroll
+                for (int e = 0; e < PR; ++e) acc[h][e] *= c;
+                if (t4 == (h & 3)) ls[h >> 2] *= c;
+            }
+            mx[h] = m;
+            if (t4 == (h & 3)) {
+                const float p0 = ok0 ? expf(s0 - m) : 0.f, p1 = ok1 ? expf(s1 - m) : 0.f;
+                ls[h >> 2] += p0 + p1;
+                ps[warp][g8][h] = p0;
+                ps[warp][g8 + 8][h] = p1;
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < kAttnTile; ++r) {
+            float v[4] = {bf_lo(vw[r].x), bf_hi(vw[r].x), bf_lo(vw[r].y), bf_hi(vw[r].y)};
+#pragma unroll
+            for (int b = 0; b < GP / 4; ++b) {
+                const float4 p4 = *reinterpret_cast<const float4*>(&ps[warp][r][4 * b]);
+                const float pp[4] = {p4.x, p4.y, p4.z, p4.w};
+#pragma unroll
+                for (int hh = 0; hh < 4; ++hh)
+                    if (4 * b + hh < G) {
+#pragma unroll
+                        for (int e = 0; e < PR; ++e) acc[4 * b + hh < G ? 4 * b + hh : 0][e] = fmaf(pp[hh], v[e], acc[4 * b + hh < G ? 4 * b + hh : 0][e]);
+                    }
             }
         }
     }
-    // merge the position groups of this warp (lanes with equal e0)
+    if (!synced) __syncthreads();
+    // merge the warps (in warp order); one without a position has maximum -inf
 #pragma unroll
-    for (int o = LPR; o < 32; o <<= 1) {
-#pragma unroll
-        for (int h = 0; h < GMAX; ++h) {
-            if (h >= G) break;
-            const float m2 = __shfl_xor_sync(0xffffffffu, mx[h], o);
-            const float l2 = __shfl_xor_sync(0xffffffffu, ls[h], o);
-            float a2[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) a2[e] = __shfl_xor_sync(0xffffffffu, acc[h][e], o);
-            const float M = fmaxf(mx[h], m2);
-            if (M != -CUDART_INF_F) {
-                const float c1 = expf(mx[h] - M), c2 = expf(m2 - M);
-                ls[h] = ls[h] * c1 + l2 * c2;
-#pragma unroll
-                for (int e = 0; e < 8; ++e) acc[h][e] = acc[h][e] * c1 + a2[e] * c2;
-                mx[h] = M;
-            }
-        }
+    for (int o = 4; o < 32; o <<= 1) {
+        ls[0] += __shfl_xor_sync(0xffffffffu, ls[0], o);
+        ls[1] += __shfl_xor_sync(0xffffffffu, ls[1], o);
     }
-    if (grp == 0) {
+    if (g8 == 0) {
+        wl[warp][t4] = ls[0];
+        wl[warp][t4 + 4] = ls[1];
+    }
 #pragma unroll
-        for (int h = 0; h < GMAX; ++h) {
-            if (h >= G) break;
-            if (lane == 0) {
-                wm[warp][h] = mx[h];
-                wl[warp][h] = ls[h];
-            }
+    for (int h = 0; h < G; ++h) {
+        if (lane == h) wm[warp][h] = mx[h];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) wacc[warp][h][e0 + e] = acc[h][e];
-        }
+        for (int e = 0; e < PR; ++e) wacc[warp][h][lane * PR + e] = acc[h][e];
     }
     __syncthreads();
-    // merge warps; write this split's partial (acc[D], m, l) per query head
-    const int S_stride = kAttnMaxSplits;
-    for (int i = threadIdx.x; i < G * D; i += blockDim.x) {
-        const int h = i / D, e = i - h * D;
-        float M = -CUDART_INF_F, L = 0.f, O = 0.f;
+    float* part = a.part + ((int64_t)g * G * kAttnMaxSplits + s) * (D + 2);
+    if (threadIdx.x < G) {
+        const int h = threadIdx.x;
+        float M = -CUDART_INF_F, L = 0.f;
+        for (int w = 0; w < NW; ++w) M = fmaxf(M, wm[w][h]);
         for (int w = 0; w < NW; ++w) {
-            const float m2 = wm[w][h];
-            const float Mn = fmaxf(M, m2);
-            if (Mn == -CUDART_INF_F) continue;
-            const float c1 = expf(M - Mn), c2 = expf(m2 - Mn);
-            L = L * c1 + wl[w][h] * c2;
-            O = O * c1 + wacc[w][h][e] * c2;
-            M = Mn;
+            const float c = wm[w][h] == -CUDART_INF_F ? 0.f : expf(wm[w][h] - M);
+            wgt[w][h] = c;
+            // (a warp whose every score was -inf poisons the sum, as exp(-inf + inf) does)
+            if (wm[w][h] != -CUDART_INF_F || wl[w][h] != 0.f) L = fmaf(c, wl[w][h], L);
         }
-        float* pp = a.part + ((int64_t)(g * G + h) * S_stride + s) * (D + 2);
-        pp[e] = O;
-        if (e == 0) {
-            pp[D] = M;
-            pp[D + 1] = L;
-        }
+        part[(int64_t)h * kAttnMaxSplits * (D + 2) + D] = M;
+        part[(int64_t)h * kAttnMaxSplits * (D + 2) + D + 1] = L;
     }
-    __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) is_last = atomicAdd(&a.ticket[g], 1) == S - 1;
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    for (int i = threadIdx.x; i < G * D; i += blockDim.x) {
+    for (int i = threadIdx.x; i < G * D; i += kAttnThreads) {
         const int h = i / D, e = i - h * D;
-        const float* base = a.part + (int64_t)(g * G + h) * S_stride * (D + 2);
-        float M = -CUDART_INF_F;
-        for (int sp = 0; sp < S; ++sp) M = fmaxf(M, __ldcg(&base[sp * (D + 2) + D]));
-        float L = 0.f, O = 0.f;
-        for (int sp = 0; sp < S; ++sp) {
-            const float ms = __ldcg(&base[sp * (D + 2) + D]);
-            if (ms == -CUDART_INF_F) continue;
-            const float c = expf(ms - M);
-            L = fmaf(__ldcg(&base[sp * (D + 2) + D + 1]), c, L);
-            O = fmaf(__ldcg(&base[sp * (D + 2) + e]), c, O);
-        }
-        a.out[(int64_t)(g * G + h) * D + e] = O / L;
+        float o = 0.f;
+#pragma unroll
+        for (int w = 0; w < NW; ++w)
+            if (wm[w][h] != -CUDART_INF_F || wl[w][h] != 0.f) o = fmaf(wgt[w][h], wacc[w][h][e], o);
+        part[(int64_t)h * kAttnMaxSplits * (D + 2) + e] = o;
     }
-    if (threadIdx.x == 0) a.ticket[g] = 0;
+}
+
+// o = sum_s w_s o_s / sum_s w_s l_s, w_s = exp(m_s - max m), of head blockIdx.x
+// and 32 dimensions from 32 blockIdx.y on; warp y takes splits y, y + 8, ...
+template <int D>
+__global__ void __launch_bounds__(256) k_attn_merge(const float* __restrict__ part, float* __restrict__ out, int S) {
+    __shared__ float red[8][32];
+    pdl_wait();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const float* base = part + (int64_t)blockIdx.x * kAttnMaxSplits * (D + 2);
+    float m[kAttnMaxSplits / 32], l[kAttnMaxSplits / 32], M = -CUDART_INF_F, L = 0.f;
+#pragma unroll
+    for (int k = 0; k < kAttnMaxSplits / 32; ++k) {
+        const int s = 32 * k + lane;
+        m[k] = s < S ? base[s * (D + 2) + D] : -CUDART_INF_F;
+        l[k] = s < S ? base[s * (D + 2) + D + 1] : 0.f;
+    }
+    float o[kAttnMaxSplits / 8];
+#pragma unroll
+    for (int k = 0; k < kAttnMaxSplits / 8; ++k)
+        o[k] = w + 8 * k < S ? base[(w + 8 * k) * (D + 2) + blockIdx.y * 32 + lane] : 0.f;
+#pragma unroll
+    for (int k = 0; k < kAttnMaxSplits / 32; ++k) M = fmaxf(M, m[k]);
+#pragma unroll
+    for (int d = 16; d; d >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, d));
+#pragma unroll
+    for (int k = 0; k < kAttnMaxSplits / 32; ++k) {
+        m[k] = m[k] == -CUDART_INF_F ? 0.f : expf(m[k] - M);
+        L = fmaf(m[k], l[k], L);
+    }
+    L = warp_sum(L);
+    float sum = 0.f;
+#pragma unroll
+    for (int k = 0; k < kAttnMaxSplits / 8; ++k) {
+        const float wt = __shfl_sync(0xffffffffu, m[k / 4], (w + 8 * k) & 31);
+        if (w + 8 * k < S && wt != 0.f) sum = fmaf(wt, o[k], sum);
+    }
+    red[w][lane] = sum;
+    __syncthreads();
+    if (w == 0) {
+        float t = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) t += red[k][lane];
+        out[blockIdx.x * D + blockIdx.y * 32 + lane] = t / L;
+    }
 }
 
 // Decode attention of one layer on a thread-block cluster per key-value head
@@ -1437,6 +1515,7 @@ __device__ __forceinline__ int float_key(float f) {
 __device__ __forceinline__ float key_float(int k) { return __int_as_float(k >= 0 ? k : k ^ 0x7fffffff); }
 
 __global__ void k_tau_init(int* scratch) {
+    pdl_launch_dependents();
     if (threadIdx.x == 0) {
         scratch[0] = float_key(INFINITY);
         scratch[1] = 0;
@@ -1624,10 +1703,33 @@ cudaError_t launch_vocab(const VocabArgs& v, int grid, bool pdl, cudaStream_t s)
     if (v.tiled) return launch_k(k_vocab, dim3(grid), dim3(kGemvThreads), smem, pdl, s, v);
     return launch_k(k_vocab_rowmajor, dim3(grid), dim3(kGemvThreads), smem, pdl, s, v);
 }
-cudaError_t launch_attention(const AttnArgs& a, int head_dim, bool pdl, cudaStream_t s) {
-    const dim3 grid(kAttnMaxSplits, a.KH);
-    if (head_dim == 64) return launch_k(k_attention<64>, grid, dim3(kAttnThreads), 0, pdl, s, a);
-    if (head_dim == 128) return launch_k(k_attention<128>, grid, dim3(kAttnThreads), 0, pdl, s, a);
+// Splits of 128 positions (a tile per warp), longer ones past kAttnMaxSplits
+// of them.
+template <int D>
+static cudaError_t launch_attention_d(const AttnArgs& a, cudaStream_t s) {
+    const int64_t per = 128;
+    const int S0 = (int)std::min<int64_t>(kAttnMaxSplits, ((int64_t)a.T + per - 1) / per);
+    const int chunk = (int)((((int64_t)a.T + S0 - 1) / S0 + kAttnTile - 1) / kAttnTile * kAttnTile);
+    const int S = (int)(((int64_t)a.T + chunk - 1) / chunk);
+    const dim3 grid(S, a.KH), block(kAttnThreads);
+    cudaError_t e = cudaErrorInvalidValue;
+    switch (a.A / a.KH) {
+        case 1: e = launch_k(k_attn_split<D, 1>, grid, block, 0, false, s, a, chunk); break;
+        case 2: e = launch_k(k_attn_split<D, 2>, grid, block, 0, false, s, a, chunk); break;
+        case 3: e = launch_k(k_attn_split<D, 3>, grid, block, 0, false, s, a, chunk); break;
+        case 4: e = launch_k(k_attn_split<D, 4>, grid, block, 0, false, s, a, chunk); break;
+        case 5: e = launch_k(k_attn_split<D, 5>, grid, block, 0, false, s, a, chunk); break;
+        case 6: e = launch_k(k_attn_split<D, 6>, grid, block, 0, false, s, a, chunk); break;
+        case 7: e = launch_k(k_attn_split<D, 7>, grid, block, 0, false, s, a, chunk); break;
+        case 8: e = launch_k(k_attn_split<D, 8>, grid, block, 0, false, s, a, chunk); break;
+        default: break;
+    }
+    if (e != cudaSuccess) return e;
+    return launch_k(k_attn_merge<D>, dim3(a.A, D / 32), dim3(256), 0, true, s, (const float*)a.part, a.out, S);
+}
+cudaError_t launch_attention(const AttnArgs& a, int head_dim, cudaStream_t s) {
+    if (head_dim == 64) return launch_attention_d<64>(a, s);
+    if (head_dim == 128) return launch_attention_d<128>(a, s);
     return cudaErrorInvalidValue;
 }
 cudaError_t launch_attention_cluster(const AttnArgs& a, int head_dim, int cluster, bool pdl, cudaStream_t s) {

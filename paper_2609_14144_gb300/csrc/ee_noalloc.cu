@@ -1,7 +1,7 @@
 // Split-K decode attention for callers that cannot allocate device memory.
 //
 // ee_attention_decode needs a caller-provided scratch buffer for its per-split
-// partial results and arrival counters.  Some callers have no way to provide
+// partial results.  Some callers have no way to provide
 // one: their device memory is owned entirely by another allocator (a serving
 // framework's pool that has reserved almost all of HBM, where an extra
 // cudaMalloc fails or fragments the pool), they run on latency-critical paths
@@ -55,7 +55,7 @@ extern "C" int ee_attention_decode_static(const float* q, const uint16_t* k_page
         return ee::set_last_error(EE_EINVAL, "bad head grouping");
     if (T <= 0 || page_size <= 0) return ee::set_last_error(EE_EINVAL, "T and page_size must be positive");
     const size_t part = align_up(4 * (size_t)n_heads * ee::kAttnMaxSplits * (head_dim + 2));
-    const size_t need = part + 4 * (size_t)n_kv_heads;
+    const size_t need = part + 4 * (size_t)n_kv_heads;  // what ee_attention_scratch_bytes asks for, unrounded
     if (need > kStaticBytes) {
         const std::string m = "this shape needs " + std::to_string(need) + " bytes of scratch but the static area holds " +
                               std::to_string(kStaticBytes) + " (n_heads * (head_dim + 2) must be at most " +
@@ -66,7 +66,6 @@ extern "C" int ee_attention_decode_static(const float* q, const uint16_t* k_page
     int rc = scratch_address(&base);
     if (rc != EE_OK) return rc;
     cudaStream_t s = (cudaStream_t)stream;
-    char* sc = (char*)base;
     ee::AttnArgs a{};
     a.q = q;
     a.kp = k_pages;
@@ -78,11 +77,8 @@ extern "C" int ee_attention_decode_static(const float* q, const uint16_t* k_page
     a.KH = n_kv_heads;
     a.page_size = page_size;
     a.out = out;
-    a.part = (float*)sc;
-    a.ticket = (int*)(sc + part);
-    // The arrival counters must start at zero; the partial sums need no clearing.
-    cudaError_t e = cudaMemsetAsync(a.ticket, 0, 4 * (size_t)n_kv_heads, s);
-    if (e == cudaSuccess) e = ee::launch_attention(a, head_dim, false, s);
+    a.part = (float*)base;  // the partial sums need no clearing
+    const cudaError_t e = ee::launch_attention(a, head_dim, s);
     if (e != cudaSuccess) return ee::set_last_error(EE_ECUDA, cudaGetErrorString(e));
     return EE_OK;
 }

@@ -52,6 +52,34 @@ def test_attention_decode(T, A, KH, D):
         assert rel_err(got[h], ref) <= 1e-4, (h, rel_err(got[h], ref))
 
 
+@pytest.mark.parametrize("G", [1, 2, 3, 4, 5, 6, 7, 8])
+@pytest.mark.parametrize("T,P,D", [(127, 64, 128), (129, 1, 64), (2065, 24, 128), (16384, 256, 64), (16401, 100, 128)])
+def test_attention_decode_groups_tiles_and_pages(T, P, D, G):
+    """Every group size at the edges of a warp's 16-position tile, of a
+    128-position split and of the split count (128 splits hold 16384), with
+    pages of any length.  The bound: products and sums in fp32, n terms of a
+    convex combination of values up to 4.5 in size, sqrt(T) rounding steps."""
+    import torch
+
+    from paper_2609_14144_gb300 import attention_decode
+
+    KH = 2
+    g = torch.Generator(device="cuda").manual_seed(T + G)
+    n_pages = (T + P - 1) // P
+    q = torch.randn(G * KH * D, generator=g, device="cuda")
+    kp = torch.randn(n_pages, KH, P, D, generator=g, device="cuda").to(torch.bfloat16)
+    vp = torch.randn(n_pages, KH, P, D, generator=g, device="cuda").to(torch.bfloat16)
+    table = torch.randperm(n_pages, generator=g, device="cuda").to(torch.int32)
+    k, v = (t[table.long()].permute(1, 0, 2, 3).reshape(KH, -1, D)[:, :T].clone() for t in (kp, vp))
+    for t in (kp, vp):  # rows past T of the last page are never read
+        used = (T - 1) % P + 1
+        t[table[-1].long(), :, used:] = float("nan")
+    got = attention_decode(q, kp, vp, table, T, G * KH, KH, D, P).view(KH, G, D)
+    ref = torch.softmax(q.double().view(KH, G, D) @ k.double().transpose(1, 2) / math.sqrt(D), -1) @ v.double()
+    err = (got.double() - ref).abs().max().item()
+    assert err <= 4.5 * math.sqrt(T) * 2.0 ** -24 * 8, err
+
+
 @pytest.mark.parametrize("V,d", [(4096, 256), (4093, 256), (151936, 896), (151937, 1536), (1000, 2048)])
 def test_vocab_confidence(V, d):
     import torch
