@@ -290,6 +290,14 @@ bool umma_available();
 int umma_splits(int64_t n_tiles, int K, int n_sm);
 cudaError_t launch_mm_umma(const uint16_t* W, int64_t n_rows, int K, const uint16_t* x3, int M, int S, float* part,
                            int Np, int* err, cudaStream_t s);
+// tcgen05 attention of a batch (ee_uattn.cu), for batches of at least
+// kUaMinRows rows: keys per split, the launch (its split outputs in the
+// warp-level kernel's layout).
+constexpr int kUaMinRows = 65;
+int uattn_keys_per_split(int t_max, int A, int M, int n_sm, int max_splits);
+cudaError_t configure_uattn();
+cudaError_t launch_uattn(const DevModel& m, int j, const float* Q, const int32_t* d_pos, int Mj, int KC, int t_max, float* part,
+                         cudaStream_t s);
 // After a batched prompt: the control block as the per-position prefill
 // leaves it before its LM head (position n).
 cudaError_t launch_rows_prefill_done(const DevModel& m, int n, cudaStream_t s);

@@ -10,8 +10,10 @@
 //   k_rows_umma / k_rows_mm   a projection: Y[row][n] = sum_k W[n][k] x[row][k]
 //   k_rows_qkv       split sum, bias, RoPE at each row's position; q kept in
 //                    fp32, k and v stored bf16 into the paged cache
-//   k_rows_fattn     causal attention of every row over the cache up to its
+//   k_rows_uattn / k_rows_fattn   causal attention of every row over the cache up to its
 //                    position on the tensor cores, keys split over CTAs
+//                    (tcgen05 for batches of at least kUaMinRows rows,
+//                    ee_uattn.cu; warp-level for fewer)
 //                    (rows of the batch at earlier positions were written by
 //                    k_rows_qkv of this layer); k_rows_amerge combines the
 //                    splits
@@ -705,6 +707,14 @@ int fa_keys_per_split(int t_max, int units, int n_sm) {
 // the O projection's input parts.
 cudaError_t launch_attn(const DevModel& m, const RowsBuf& b, int j, int Mj, const int32_t* d_pos, int t_max,
                         cudaStream_t s) {
+    if (b.umma && Mj >= kUaMinRows) {
+        const int KC = uattn_keys_per_split(t_max, m.A, Mj, b.n_sm, kFaMaxSplits);
+        RCKA(launch_uattn(m, j, b.Q, d_pos, Mj, KC, t_max, b.part, s));
+        if (m.D == 128)
+            return launch_pdl(k_rows_amerge<128>, dim3(m.A, Mj), dim3(128), 0, s, m, (const float*)b.part, d_pos, KC,
+                              parts(b, Mj));
+        return launch_pdl(k_rows_amerge<64>, dim3(m.A, Mj), dim3(64), 0, s, m, (const float*)b.part, d_pos, KC, parts(b, Mj));
+    }
     const int row_blocks = (Mj + kFaWarps * 16 - 1) / (kFaWarps * 16);
     const int KC = fa_keys_per_split(t_max, m.A * row_blocks, b.n_sm);
     const int S = (t_max + KC - 1) / KC;

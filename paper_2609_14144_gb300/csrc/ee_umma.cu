@@ -44,6 +44,7 @@
 #include <mutex>
 
 #include "ee_internal.h"
+#include "ee_umma.cuh"
 
 namespace ee {
 namespace {
@@ -56,80 +57,6 @@ constexpr int kUABytes = kUMRows * kUKStage * 2;    // 8 KB
 constexpr int kUBBytes = kUKStage / 8 * 3 * kRowsMax * 16;  // a full batch's activations: 48 KB
 constexpr int kUStageBytes = kUABytes + kUBBytes;   // 56 KB
 constexpr int kUTmemCols = 2 * kRowsMax;            // two accumulators of one fp32 column per position
-constexpr long long kUWaitCycles = 4000000000ll;   // about 2 s
-
-__device__ __forceinline__ uint32_t u_saddr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void u_mb_init(uint64_t* b, int n) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(u_saddr(b)), "r"(n) : "memory");
-}
-__device__ __forceinline__ bool u_mb_test(uint64_t* b, int parity) {
-    uint32_t ok;
-    asm volatile(
-        "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-        : "=r"(ok)
-        : "r"(u_saddr(b)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// Wait for the phase of parity `parity`; false after the bound, or (when
-// `err` is given) once the error word carries kErrStall.
-__device__ __forceinline__ bool u_mb_wait(uint64_t* b, int parity, const volatile int* err) {
-    if (u_mb_test(b, parity)) return true;
-    const long long t0 = clock64();
-    for (unsigned it = 1;; ++it) {
-        if (u_mb_test(b, parity)) return true;
-        if ((it & 255) == 0) {
-            if (clock64() - t0 > kUWaitCycles) return false;
-            if (err && (*err & kErrStall)) return false;
-        }
-    }
-}
-
-// ---------------------------------------------------------------- tcgen05
-// Shared-memory operand descriptor: start address, leading (K-direction) and
-// stride (row-direction) byte offsets of the core matrices, no swizzle.
-__device__ __forceinline__ uint64_t u_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr >> 4) & 0x3fffu);
-    d |= (uint64_t)((lbo >> 4) & 0x3fffu) << 16;
-    d |= (uint64_t)((sbo >> 4) & 0x3fffu) << 32;
-    d |= (uint64_t)1 << 46;  // descriptor version of sm_100 and later
-    return d;                // base offset 0, layout type 0 (no swizzle)
-}
-// Instruction descriptor of kind::f16: fp32 accumulator, bf16 A and B, both
-// K-major, M = kUMRows, N = n (a multiple of 16, 16 <= n <= 256).
-__device__ __forceinline__ uint32_t u_idesc(int n) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kUMRows >> 4) << 24);
-}
-
-__device__ __forceinline__ void u_mma(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{ .reg .pred p; setp.ne.u32 p, %4, 0; tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p; }" ::"r"(
-            tmem_d),
-        "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-__device__ __forceinline__ void u_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(u_saddr(bar))
-                 : "memory");
-}
-__device__ __forceinline__ void u_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void u_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-
-// 16 consecutive fp32 columns of this thread's tensor-memory lane.
-__device__ __forceinline__ void u_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
 
 // ---------------------------------------------------------------- copies
 __device__ __forceinline__ void u_expect_tx(uint64_t* bar, uint32_t bytes) {
@@ -327,7 +254,8 @@ bool umma_available() {
         static uint16_t dummy[64 * 8] __attribute__((aligned(16)));
         ok = major == 10 && encode_fn() && weight_map(&probe, dummy, 4, 64) &&
              cudaFuncSetAttribute(k_rows_umma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)umma_smem()) ==
-                 cudaSuccess;
+                 cudaSuccess &&
+             configure_uattn() == cudaSuccess;
         cudaGetLastError();
     }
     return ok == 1;

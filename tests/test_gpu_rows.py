@@ -110,6 +110,36 @@ def test_tiny_prompt_paths_agree(tiny_model):
         tok = rb["token"]
 
 
+@pytest.mark.parametrize("D,page", [(64, 16), (64, 256), (128, 64), (128, 32)])
+@pytest.mark.parametrize("n", [64, 65, 127, 129, 193, 700])
+def test_tcgen05_attention_row_and_key_edges(n, D, page):
+    """The batched attention at the edges of its row tile (128 rows, from 65
+    on), of a block of 64 keys and of a key split, with pages shorter and
+    longer than a block in any order, seven query heads to a key-value head:
+    against the same prompt one position at a time (fp32 path)."""
+    from paper_2609_14144_gb300 import OPT_DEBUG_LOGITS, OPT_ROWS, Engine
+
+    shape = TINY.replace(n_heads=14, head_dim=D, n_layers=2, readout_layers=(1,))
+    model = synth.make_model(shape)
+    pages = np.random.default_rng(n).permutation((n + 1 + page - 1) // page).astype(np.int32)
+    prompt = synth.token_ids(shape.seed, 905, n, shape.vocab)
+    got = []
+    for rows in (1, 0):
+        eng = Engine(shape, model, max_ctx=n + 1, page_size=page)
+        eng.set_option(OPT_ROWS, rows)
+        eng.set_option(OPT_DEBUG_LOGITS, 1)
+        eng.set_page_table(pages)
+        eng.prefill(prompt)
+        got.append(eng)
+    a, b = got
+    assert rel_err(a.hidden_final(), b.hidden_final()) <= PATH_TOL
+    assert rel_err(a.final_logits(), b.final_logits()) <= PATH_TOL
+    for t in sorted({0, 1, 62, 63, n // 2, n - 66, n - 2, n - 1}):
+        if 0 <= t < n:  # layer 1's entries carry layer 0's attention of that row
+            for x, y in zip(a.kv(1, t), b.kv(1, t)):
+                assert rel_err(x, y) <= REL_TOL, t
+
+
 def _exit_decode(shape, model, n, force_of, rows=True):
     P = shape.prompt_len
     orc = oracle.Oracle(shape, model, max_ctx=P + n + 1)
