@@ -50,7 +50,7 @@ WORKLOAD = "1.5b"
 HEADLINE_RATE = 0.5
 CALIB_TOKENS = 2048
 REPASS_W = 16  # positions in the measured full-depth re-pass
-ROWS_MAX = 256  # positions per batch of the multi-position layer pass (EE_OPT_ROWS)
+ROWS_MAX = 1024  # positions per batch of the multi-position layer pass (EE_OPT_ROWS)
 CTL_BYTES = 368  # device control block read back by a host-buffer ee_decode_n
 
 
@@ -758,12 +758,12 @@ def rows_launches(L: int, M: int, kv_only: bool) -> int:
 
 def profile_rows(shape, model, local: int):
     """--profile-run --rows: the multi-position layer pass for ncu captures.
-    A 256-position prompt in two batches, 16 exit steps (direct launches),
+    A 512-position prompt in one batch, 16 exit steps (direct launches),
     then one re-pass of those 16 positions in one batch.  Prints the launch
     counts of each part."""
     from paper_2609_14144_gb300 import DEVICE, FORCE_EXIT_AT, OPT_GRAPHS, OPT_ROWS, Engine
 
-    P, n = 2 * ROWS_MAX, REPASS_W
+    P, n = 512, REPASS_W
     eng = Engine(shape, model, max_ctx=P + n, device=local)
     eng.set_option(OPT_GRAPHS, 0)
     eng.set_option(OPT_ROWS, 1)
@@ -772,7 +772,7 @@ def profile_rows(shape, model, local: int):
     eng.sync()
     n_rp = eng.repass(P, P + n)
     L, k = shape.n_layers, shape.readout_layers[0]
-    prefill = rows_launches(L, ROWS_MAX, True) + rows_launches(L, P - ROWS_MAX, False) + 4
+    prefill = rows_launches(L, P, False) + 4
     decode = sum(step_launches(L, shape.readout_layers, 0, eng.persistent) for _ in range(n)) + 1
     repass = rows_launches(L - k, n, False)
     print(json.dumps({"prefill_launches": prefill, "decode_launches": decode, "repass_launches": repass,

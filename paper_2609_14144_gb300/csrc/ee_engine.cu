@@ -634,25 +634,27 @@ int rows_repass(ee_ctx* c, const std::vector<int32_t>& todo, const std::vector<i
         const int M = std::min(kRowsMax, n - b0);
         const bool last = b0 + M == n;
         const int t_max = *std::max_element(pos.begin() + b0, pos.begin() + b0 + M) + 1;
-        EE_CK(rows_pass(m, c->rows, start.data() + b0, M, d_pos + b0, nullptr, 0, t_max, !last, s));
+        EE_CK(rows_pass(m, c->rows, start.data() + b0, M, d_pos + b0, nullptr, 0, t_max, last ? last_row : -1, s));
     }
     EE_CK(cudaMemcpyAsync(m.h, c->rows.H + (int64_t)last_row * m.d, 4 * (size_t)m.d, cudaMemcpyDeviceToDevice, s));
     EE_TRY(fetch_ctl(c));
     return device_error(c);
 }
 
-// The prompt in batches of kRowsMax positions through the multi-position
-// layer pass (only the last batch runs the last layer past its cache
-// entries), then the LM head on the last position's final residual.
+// The prompt in as few batches of at most kRowsMax positions as hold it, of
+// equal size, through the multi-position layer pass (only the last position
+// runs the last layer past its cache entries), then the LM head on its final
+// residual.
 int rows_prefill(ee_ctx* c, const int32_t* d_prompt, int n) {
     cudaStream_t s = c->stream;
     const DevModel& m = c->dm;
     const std::vector<int> start(kRowsMax, 0);
     int last_row = 0;
-    for (int b0 = 0; b0 < n; b0 += kRowsMax) {
-        const int M = std::min(kRowsMax, n - b0);
-        EE_CK(rows_pass(m, c->rows, start.data(), M, c->rows.pos, d_prompt + b0, b0, b0 + M, b0 + M < n, s));
+    const int batches = (n + kRowsMax - 1) / kRowsMax, size = (n + batches - 1) / batches;
+    for (int b0 = 0; b0 < n; b0 += size) {
+        const int M = std::min(size, n - b0);
         last_row = M - 1;
+        EE_CK(rows_pass(m, c->rows, start.data(), M, c->rows.pos, d_prompt + b0, b0, b0 + M, b0 + M < n ? -1 : last_row, s));
     }
     EE_CK(cudaMemcpyAsync(m.h, c->rows.H + (int64_t)last_row * m.d, 4 * (size_t)m.d, cudaMemcpyDeviceToDevice, s));
     EE_CK(launch_rows_prefill_done(m, n, s));

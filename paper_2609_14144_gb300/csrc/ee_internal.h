@@ -251,16 +251,22 @@ cudaError_t launch_vocab_ring(const VocabArgs& v, const VocabRing& vr, bool pdl,
 // each layer over up to kRowsMax positions at once, every weight byte read
 // once per batch.  Products are tensor-core mma of the bf16 weights with the
 // fp32 activations split into three bf16 parts (high, middle, low).
-constexpr int kRowsMax = 256;            // positions per batch (the tcgen05 products' largest N)
-// Row stride of a batch's activation parts: M rounded up to 16.
-__host__ __device__ constexpr int x3_rows(int M) { return (M + 15) & ~15; }
+constexpr int kRowsMax = 1024;           // positions per batch
+constexpr int kRowsBlock = 256;          // rows of one tcgen05 product (at most: its largest N)
+// Rows of each block of a batch of M rows: as few blocks of at most kRowsBlock
+// rows as hold it, of equal size up to a multiple of 16.  (Equal, so that a
+// few rows past a full block do not leave CTAs with a block of their own.)
+__host__ __device__ constexpr int rows_blocks(int M) { return (M + kRowsBlock - 1) / kRowsBlock; }
+__host__ __device__ constexpr int x3_rows(int M) {
+    return ((M + rows_blocks(M) - 1) / rows_blocks(M) + 15) & ~15;
+}
 constexpr int kRowsTargetUnits = 2432;   // (tile, K split) units a projection aims for: 152 SMs x 16 warps
 struct RowsBuf {
     float* H;           // [kRowsMax][d] residual of each row
     uint16_t* x3;       // next product's input as three bf16 parts (high, x - high, the rest),
-                        // chunk-major: [ldx / 8][3][x3_rows(M)][8] for a batch of M rows
+                        // chunk-major: [blocks][ldx / 8][3][x3_rows(M)][8] for a batch of M rows
     float* Q;           // [kRowsMax][A D] rotated queries
-    float* part;        // split partials [S][M][n_rows padded to 32]
+    float* part;        // split partials [S][M][n_rows padded to 32] of a projection, [S][M][A][D + 2] of the attention
     int32_t* pos;       // [kRowsMax] positions of a prompt batch
     int64_t part_floats;
     int ldx;
@@ -278,17 +284,18 @@ int64_t rows_part_floats(int d, int A, int KH, int D, int F);
 // start): row i starts at layer start[i] (host, non-decreasing).  With ids,
 // rows take the embedding of ids[i] and positions pos_base + i (written to
 // d_pos); otherwise each row starts from h_exit at its position.  t_max:
-// the largest position of the batch + 1.  kv_only: the last layer stops
-// after its cache entries.
+// the largest position of the batch + 1.  last_row: the one row whose final
+// residual is wanted (in H), -1 for none; the other rows' last layer stops
+// after its cache entries, which is all that anything reads of it.
 cudaError_t rows_pass(const DevModel& m, const RowsBuf& b, const int* start, int M, int32_t* d_pos,
-                      const int32_t* ids, int pos_base, int t_max, bool kv_only, cudaStream_t s);
+                      const int32_t* ids, int pos_base, int t_max, int last_row, cudaStream_t s);
 // tcgen05 projections of the multi-position pass (ee_umma.cu): available on
 // this device (tensor-map encoding and the kernel's shared memory), the K
 // splits for n_sm SMs, and one projection into part[S][M][Np] (the layout of
 // the warp-level path).
 bool umma_available();
-int umma_splits(int64_t n_tiles, int K, int n_sm);
-cudaError_t launch_mm_umma(const uint16_t* W, int64_t n_rows, int K, const uint16_t* x3, int M, int S, float* part,
+int umma_splits(int64_t n_tiles, int K, int M, int n_sm);
+cudaError_t launch_mm_umma(const uint16_t* W, int64_t n_rows, int K, const uint16_t* x3, int ldx, int M, int S, float* part,
                            int Np, int* err, cudaStream_t s);
 // tcgen05 attention of a batch (ee_uattn.cu), for batches of at least
 // kUaMinRows rows: keys per split, the launch (its split outputs in the

@@ -54,21 +54,22 @@ constexpr int kRowsWarps = kRowsThreads / 32;
 __device__ __forceinline__ float r_bf2f(uint16_t b) { return __uint_as_float((uint32_t)b << 16); }
 __device__ __forceinline__ uint16_t r_f2bf(float f) { return __bfloat16_as_ushort(__float2bfloat16_rn(f)); }
 
-// A product's input as three bf16 parts, stored chunk-major: for each
-// 16-byte column chunk (8 columns), the high parts of the batch's rows, then
-// the middle parts, then the low parts, 16 bytes per row and `rows` rows a
-// part (the batch's row count rounded up to 16).  One part of a chunk is then
+// A product's input as three bf16 parts, stored chunk-major in blocks of
+// `rows` rows (x3_rows of the batch): for each 16-byte column chunk (8
+// columns) of a block, the high parts of its rows, then the middle parts, then
+// the low parts, 16 bytes per row.  One part of a chunk is then
 // the tensor cores' operand of N = rows rows in their canonical layout
 // (ee_umma.cu), a few chunks one contiguous stage whatever the batch size,
 // and a warp-level product reads a row's chunk of one part as 16 contiguous
 // bytes.
 struct Parts {
     uint16_t* p;
-    int rows;
+    int rows, ldx;
+    __device__ __forceinline__ int64_t index(int part, int row, int col) const {
+        const int b = row / rows;
+        return ((((int64_t)b * (ldx >> 3) + (col >> 3)) * 3 + part) * rows + (row - b * rows)) * 8 + (col & 7);
+    }
 };
-__device__ __forceinline__ int64_t x3_index(int part, int row, int col, int rows) {
-    return (((int64_t)(col >> 3) * 3 + part) * rows + row) * 8 + (col & 7);
-}
 
 // The three bf16 parts of x at (row, col): high = bf16(x), middle = bf16(x -
 // high), low = bf16(x - high - middle) (each difference exact in fp32).
@@ -76,9 +77,10 @@ __device__ __forceinline__ void split_store(float x, const Parts& p, int row, in
     const uint16_t h = r_f2bf(x);
     const float r1 = x - r_bf2f(h);
     const uint16_t md = r_f2bf(r1);
-    p.p[x3_index(0, row, col, p.rows)] = h;
-    p.p[x3_index(1, row, col, p.rows)] = md;
-    p.p[x3_index(2, row, col, p.rows)] = r_f2bf(r1 - r_bf2f(md));
+    const int64_t at = p.index(0, row, col);
+    p.p[at] = h;
+    p.p[at + p.rows * 8] = md;
+    p.p[at + p.rows * 16] = r_f2bf(r1 - r_bf2f(md));
 }
 // Columns from n up to the next multiple of 64 (a tensor-core stage) read as 0.
 __host__ __device__ __forceinline__ int pad64(int n) { return (n + 63) & ~63; }
@@ -173,7 +175,7 @@ __global__ void __launch_bounds__(kRowsThreads) k_rows_mm(const uint4* __restric
                 for (int n = 0; n < NB; ++n) {
                     const int row = r0 + n * 8 + g;
                     const bool okx = ok && row < M;
-                    const uint16_t* at = x3.p + x3_index(0, okx ? row : 0, ch * 8, x3.rows);
+                    const uint16_t* at = x3.p + x3.index(0, okx ? row : 0, ch * 8);
                     bh[v][n] = okx ? ld_act(at) : make_uint4(0u, 0u, 0u, 0u);
                     bm[v][n] = okx ? ld_act(at + x3.rows * 8) : make_uint4(0u, 0u, 0u, 0u);
                     bl[v][n] = okx ? ld_act(at + 2 * x3.rows * 8) : make_uint4(0u, 0u, 0u, 0u);
@@ -601,10 +603,10 @@ __global__ void __launch_bounds__(kFaThreads) k_rows_fattn(DevModel m, int j, co
     }
     if (!act) return;
     // the split's unnormalised output, maximum and sum of each row:
-    // part[((s kRowsMax + row) A + h)][D + 2]
+    // part[((s Mj + row) A + h)][D + 2]
     const int ld = D + 2;
-    float* q0 = part + ((int64_t)(s * kRowsMax + r0) * m.A + h) * ld;
-    float* q1 = part + ((int64_t)(s * kRowsMax + r1) * m.A + h) * ld;
+    float* q0 = part + ((int64_t)(s * Mj + r0) * m.A + h) * ld;
+    float* q1 = part + ((int64_t)(s * Mj + r1) * m.A + h) * ld;
 #pragma unroll
     for (int n = 0; n < NT; ++n) {
         const int c = n * 8 + 2 * t4;
@@ -640,7 +642,7 @@ __global__ void __launch_bounds__(D) k_rows_amerge(DevModel m, const float* __re
     const int h = blockIdx.x, i = blockIdx.y, e = threadIdx.x;
     const int ns = pos[i] / KC + 1, ld = D + 2;
     const float* q = part + ((int64_t)i * m.A + h) * ld;
-    const int64_t step = (int64_t)kRowsMax * m.A * ld;  // one split
+    const int64_t step = (int64_t)gridDim.y * m.A * ld;  // one split
     float M = -INFINITY;
     for (int s = 0; s < ns; ++s) M = fmaxf(M, q[s * step + D]);
     float num = 0.f, den = 0.f;
@@ -672,9 +674,9 @@ cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t sme
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
-// The activation parts of a batch of M rows (row stride M rounded up to 16,
-// the operand rows of the tensor-core products).
-Parts parts(const RowsBuf& b, int M) { return Parts{b.x3, x3_rows(M)}; }
+// The activation parts of a batch of M rows (in blocks of x3_rows(M), the
+// operand rows of the tensor-core products).
+Parts parts(const RowsBuf& b, int M) { return Parts{b.x3, x3_rows(M), b.ldx}; }
 
 #define RCKA(x)                                   \
     do {                                          \
@@ -695,20 +697,23 @@ void row_groups(int M, int& NB, int& RG) {
 // resident per SM: its stages take over half the shared memory), and at most
 // kFaMaxSplits.  (Two or four waves of shorter splits were slower: every
 // split is a partial result written, merged and read again.)
-int fa_keys_per_split(int t_max, int units, int n_sm) {
-    const int target = std::max(1, std::min(kFaMaxSplits, n_sm / std::max(1, units)));
+int fa_keys_per_split(int t_max, int units, int n_sm, int max_splits) {
+    const int target = std::max(1, std::min(max_splits, n_sm / std::max(1, units)));
     int kc = (t_max + target - 1) / target;
     kc = std::max(kFaKeys, (kc + kFaKeys - 1) / kFaKeys * kFaKeys);
-    while ((t_max + kc - 1) / kc > kFaMaxSplits) kc += kFaKeys;
+    while ((t_max + kc - 1) / kc > max_splits) kc += kFaKeys;
     return kc;
 }
+// Key splits of a batch of M rows (at most): their partial results fit what
+// kFaMaxSplits splits of kRowsBlock rows take.
+int attn_splits(int M) { return std::max(1, std::min(kFaMaxSplits, kFaMaxSplits * kRowsBlock / M)); }
 
 // The batch's attention at layer j: the split kernel, then the merge into
 // the O projection's input parts.
 cudaError_t launch_attn(const DevModel& m, const RowsBuf& b, int j, int Mj, const int32_t* d_pos, int t_max,
                         cudaStream_t s) {
     if (b.umma && Mj >= kUaMinRows) {
-        const int KC = uattn_keys_per_split(t_max, m.A, Mj, b.n_sm, kFaMaxSplits);
+        const int KC = uattn_keys_per_split(t_max, m.A, Mj, b.n_sm, attn_splits(Mj));
         RCKA(launch_uattn(m, j, b.Q, d_pos, Mj, KC, t_max, b.part, s));
         if (m.D == 128)
             return launch_pdl(k_rows_amerge<128>, dim3(m.A, Mj), dim3(128), 0, s, m, (const float*)b.part, d_pos, KC,
@@ -716,7 +721,7 @@ cudaError_t launch_attn(const DevModel& m, const RowsBuf& b, int j, int Mj, cons
         return launch_pdl(k_rows_amerge<64>, dim3(m.A, Mj), dim3(64), 0, s, m, (const float*)b.part, d_pos, KC, parts(b, Mj));
     }
     const int row_blocks = (Mj + kFaWarps * 16 - 1) / (kFaWarps * 16);
-    const int KC = fa_keys_per_split(t_max, m.A * row_blocks, b.n_sm);
+    const int KC = fa_keys_per_split(t_max, m.A * row_blocks, b.n_sm, attn_splits(Mj));
     const int S = (t_max + KC - 1) / KC;
     const dim3 grid(m.KH, S, (m.A / m.KH) * row_blocks);
     if (m.D == 128) {
@@ -738,9 +743,9 @@ cudaError_t launch_mm(const uint16_t* W, int64_t n_rows, int K, const RowsBuf& b
     const int64_t nt = tile_count(n_rows);
     if (b.umma) {
         Np = (int)(nt * kTileRows);
-        S = umma_splits(nt, K, b.n_sm);
+        S = umma_splits(nt, K, M, b.n_sm);
         S = (int)std::max<int64_t>(1, std::min<int64_t>(S, b.part_floats / ((int64_t)M * Np)));
-        return launch_mm_umma(W, n_rows, K, b.x3, M, S, b.part, Np, b.err, s);
+        return launch_mm_umma(W, n_rows, K, b.x3, b.ldx, M, S, b.part, Np, b.err, s);
     }
     int NB, RG;
     row_groups(M, NB, RG);
@@ -797,8 +802,8 @@ int64_t rows_part_floats(int d, int A, int KH, int D, int F) {
             const int64_t nt = tile_count(rows[p]);
             most = std::max(most, (int64_t)rows_splits(nt, K[p], M) * M * nt * kTileRows);
         }
-    // the flash attention's split outputs: [kFaMaxSplits][kRowsMax][A][D + 2]
-    return std::max(most, (int64_t)kFaMaxSplits * kRowsMax * A * (D + 2));
+    // the attention's split outputs: [attn_splits(M)][M][A][D + 2]
+    return std::max(most, (int64_t)kFaMaxSplits * kRowsBlock * A * (D + 2));
 }
 
 #define RCK(x)                                    \
@@ -807,8 +812,8 @@ int64_t rows_part_floats(int d, int A, int KH, int D, int F) {
         if (e_ != cudaSuccess) return e_;         \
     } while (0)
 
-cudaError_t rows_pass(const DevModel& m, const RowsBuf& b, const int* start, int M, int32_t* d_pos,
-                      const int32_t* ids, int pos_base, int t_max, bool kv_only, cudaStream_t s) {
+cudaError_t rows_pass(const DevModel& m, const RowsBuf& b_in, const int* start, int M, int32_t* d_pos,
+                      const int32_t* ids, int pos_base, int t_max, int last_row, cudaStream_t s) {
     if (M <= 0) return cudaSuccess;
     if (t_max <= 0 || t_max > m.max_ctx) return cudaErrorInvalidValue;
     if (M > kRowsMax || start[0] < 0 || start[M - 1] >= m.L) return cudaErrorInvalidValue;
@@ -816,6 +821,8 @@ cudaError_t rows_pass(const DevModel& m, const RowsBuf& b, const int* start, int
         if (start[i] < start[i - 1]) return cudaErrorInvalidValue;
     const int L = m.L, d = m.d, AD = m.A * m.D;
     const int64_t nqkv = (int64_t)(m.A + 2 * m.KH) * m.D;
+    if (last_row >= M) return cudaErrorInvalidValue;
+    RowsBuf b = b_in;
     RCK(launch_pdl(k_rows_init, dim3(M), dim3(kRowsThreads), 0, s, m, b.H, d_pos, ids, pos_base));
     int M_prev = 0, S_prev = 1, Np_prev = 0;
     for (int j = start[0]; j < L; ++j) {
@@ -830,7 +837,15 @@ cudaError_t rows_pass(const DevModel& m, const RowsBuf& b, const int* start, int
         const int nu = (int)(nqkv / 2);
         RCK(launch_pdl(k_rows_qkv, dim3((nu + kRowsThreads - 1) / kRowsThreads, Mj), dim3(kRowsThreads), 0, s, m, j,
                        (const float*)b.part, S, Mj, Np, (const int32_t*)d_pos, b.Q));
-        if (kv_only && j == L - 1) return cudaSuccess;
+        if (j == L - 1) {
+            // every row's cache entries are there; what is left of the last
+            // layer is for the row whose final residual is wanted
+            if (last_row < 0) return cudaSuccess;
+            b.H += (int64_t)last_row * d;
+            b.Q += (int64_t)last_row * AD;
+            d_pos += last_row;
+            Mj = 1;
+        }
         RCK(launch_attn(m, b, j, Mj, d_pos, t_max, s));
         RCK(launch_mm(lw + m.off_wo, d, AD, b, Mj, S, Np, s));
         RCK(launch_pdl(k_rows_add_norm, dim3(Mj), dim3(kNormThreads), 0, s, b.H, d, (const float*)b.part, S, Mj, Np,

@@ -327,12 +327,12 @@ __global__ void __launch_bounds__(kUaThreads, 1)
         if (*everr & kErrStall) u_mb_wait(pv_done, (nb - 1) & 1, nullptr);  // products in flight end
         add_products();
         ua_wait_group<0>();
-        // the split's unnormalised output, maximum and sum: part[((s kRowsMax + row) A + h)][D + 2]
+        // the split's unnormalised output, maximum and sum: part[((s Mj + row) A + h)][D + 2]
         __syncthreads();
         xch[qt * kUaRows + row] = l;
         __syncthreads();
         if (my_pos >= k0) {
-            float* out = part + ((int64_t)(s * kRowsMax + r0 + row) * m.A + h) * (D + 2);
+            float* out = part + ((int64_t)(s * Mj + r0 + row) * m.A + h) * (D + 2);
 #pragma unroll
             for (int i = 0; i < HC; i += 2) *reinterpret_cast<float2*>(out + qt * HC + i) = make_float2(o[i], o[i + 1]);
             float lt = 0.f;
@@ -348,13 +348,24 @@ __global__ void __launch_bounds__(kUaThreads, 1)
 
 }  // namespace
 
-// Keys per split: a multiple of the block such that the splits, times the
-// (head, row tile) pairs, make about one wave of CTAs (one resident per SM).
+// Keys per split: a multiple of the block, the split count that needs the
+// least time by a simple count: the waves of CTAs (one resident per SM) times
+// a CTA's blocks and its set-up and write-out (about two blocks' time; four
+// more for a split beyond the first, which the merge reads back).
 int uattn_keys_per_split(int t_max, int A, int M, int n_sm, int max_splits) {
-    const int units = A * ((M + kUaRows - 1) / kUaRows);
-    const int target = std::max(1, std::min(max_splits, n_sm / std::max(1, units)));
-    const int per = (t_max + target - 1) / target;
-    return std::max(kUaKeys, (per + kUaKeys - 1) / kUaKeys * kUaKeys);
+    const int units = A * ((M + kUaRows - 1) / kUaRows), blocks = (t_max + kUaKeys - 1) / kUaKeys;
+    int best = blocks;
+    int64_t least = INT64_MAX;
+    for (int S = 1; S <= std::min(max_splits, blocks); ++S) {
+        const int per = (blocks + S - 1) / S, n = (blocks + per - 1) / per;
+        const int64_t waves = ((int64_t)units * n + n_sm - 1) / n_sm;
+        const int64_t t = 2 * waves * (per + 2) + n;
+        if (t < least) {
+            least = t;
+            best = per;
+        }
+    }
+    return best * kUaKeys;
 }
 
 cudaError_t configure_uattn() {

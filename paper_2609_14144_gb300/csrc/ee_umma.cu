@@ -3,20 +3,21 @@
 // with operands staged in shared memory by TMA and the fp32 accumulator in
 // tensor memory.
 //
-// One projection of a batch of M <= 256 positions: Y[row][n] = sum_k W[n][k]
+// One projection of a batch of positions: Y[row][n] = sum_k W[n][k]
 // x[row][k] for the n_rows x K tile-packed bf16 weights W.  Each activation
 // is carried as three bf16 parts (x = high + middle + low, ee_rows.cu), each
-// part of the batch stored as N operand rows; every K = 16 step issues
-// three MMAs of shape M = 128 (weight rows) x N (the batch's rows rounded up
-// to 16), one per part, into two fp32 accumulators whose column is the batch
+// part of a block of at most 256 of the batch's rows stored as N operand rows;
+// every K = 16 step issues three MMAs of shape M = 128 (weight rows) x N (the
+// block's rows rounded up to 16), one per part, into two fp32 accumulators whose column is the batch
 // row: the high parts' products into the first, the middle and low parts'
 // (2^-8 of the size and less) into the second, so that their small terms are
 // not added into the large sum step by step; the epilogue adds the two.  The
 // bf16 products are exact.
 //
-// CTA (x, s): weight rows [128 x, 128 x + 128) (four 32-row tiles) over the
-// K range of split s, 32 columns per pipeline stage, four stages in flight:
-//   - warp 0, lane 0 loads a stage: the 128 x 32 weight block with one TMA
+// CTA (x, s, z): weight rows [128 x, 128 x + 128) (four 32-row tiles) over the
+// K range of split s for row block z, 32 columns per pipeline stage, four
+// stages in flight:
+//   - the producer warp's lane 0 loads a stage: the 128 x 32 weight block with one TMA
 //     tensor copy (a three-dimensional view of the tile-packed layout whose
 //     box lands in shared memory in the UMMA canonical K-major layout with
 //     no swizzle: 8-row x 16-byte core matrices, 128 bytes apart along the
@@ -25,12 +26,20 @@
 //     stage is one contiguous range in the same canonical layout: a part's N
 //     rows N x 16 bytes long, the three parts of a chunk side by side, chunks
 //     3 N x 16 bytes apart along K; 48 KB for a full batch);
-//   - warp 1, lane 0 issues six MMAs per stage into the tensor-memory
+//   - the MMA warp's lane 0 issues six MMAs per stage into the tensor-memory
 //     accumulators and commits each stage back to its producer barrier;
-//   - after the last stage all four warps read the accumulators (warp w holds
-//     tensor-memory lanes 32 w .. 32 w + 31, the weight rows of tile w) and
-//     write the split's partial sums part[s][row][n], which the consumer adds
-//     in split order as with the warp-level path.
+//   - the epilogue warps read the accumulators (warps w and w + 4 hold
+//     tensor-memory lanes 32 w .. 32 w + 31, the weight rows of tile w, half of
+//     the columns each): the high parts' after every chain of stages, added to
+//     running sums in registers, both after the last stage, when they write the
+//     split's partial sums part[s][row][n], which the consumer adds in split
+//     order as with the warp-level path.
+// The tensor core adds with truncation, so the error of a sum grows with the
+// number of steps it is carried through: with a whole K range in one chain a
+// 4099-position prompt was 2.0e-4 from 64 bits in its final state, with chains
+// of 4 stages 2.5e-5.  Reading a chain back costs little tensor time: the next
+// two stages' middle and low parts' products are issued first and run under it
+// (gate/up of an 820-row batch at 3B: 162 us, 145 us in one chain).
 // Every wait is bounded; after a wait runs out the kernel flags kErrStall in
 // the device error word, waits (bounded, whatever the word says) for its
 // copies in flight and for the MMAs it issued, frees its tensor memory and
@@ -49,14 +58,27 @@
 namespace ee {
 namespace {
 
-constexpr int kUThreads = 128;
+// A launch's shape.  EW epilogue warps read the accumulators (warp w:
+// tensor-memory lanes 32 (w mod 4), columns from HC (w / 4) on), then come the
+// producer warp and the MMA warp; CH stages of the high parts' products (at
+// most) add up in tensor memory.
+template <int EW_, int HC_, int CH_>
+struct UShape {
+    static constexpr int EW = EW_, HC = HC_, CH = CH_;
+    static constexpr int threads = 32 * (EW + 2);
+};
+using ULarge = UShape<8, kRowsBlock / 2, 4>;
+// A small batch: fewer threads and registers, so that the launches before and
+// after find room beside it (programmatic launch), and longer chains, since its
+// products are too short to run under a read-back.
+using USmall = UShape<4, 64, 24>;
 constexpr int kUStages = 4;
 constexpr int kUMRows = 128;                        // weight rows per CTA (UMMA M)
 constexpr int kUKStage = 32;                        // K columns per stage
 constexpr int kUABytes = kUMRows * kUKStage * 2;    // 8 KB
-constexpr int kUBBytes = kUKStage / 8 * 3 * kRowsMax * 16;  // a full batch's activations: 48 KB
+constexpr int kUBBytes = kUKStage / 8 * 3 * kRowsBlock * 16;  // a full block's activations: 48 KB
 constexpr int kUStageBytes = kUABytes + kUBBytes;   // 56 KB
-constexpr int kUTmemCols = 2 * kRowsMax;            // two accumulators of one fp32 column per position
+constexpr int kUTmemCols = 2 * kRowsBlock;          // two accumulators of one fp32 column per position
 
 // ---------------------------------------------------------------- copies
 __device__ __forceinline__ void u_expect_tx(uint64_t* bar, uint32_t bytes) {
@@ -79,23 +101,28 @@ __device__ __forceinline__ void u_bulk(void* dst, const void* src, uint32_t byte
                  : "memory");
 }
 
-__global__ void __launch_bounds__(kUThreads, 1)
-    k_rows_umma(const __grid_constant__ CUtensorMap wmap, const uint16_t* __restrict__ x3, int n_tiles, int K, int M,
-                int S, float* __restrict__ part, int Np, int* err) {
+template <class U>
+__global__ void __launch_bounds__(U::threads, 1)
+    k_rows_umma(const __grid_constant__ CUtensorMap wmap, const uint16_t* __restrict__ x3, int ldx, int n_tiles, int K,
+                int M_all, int S, float* __restrict__ part, int Np, int* err) {
     extern __shared__ __align__(1024) uint8_t u_smem_raw[];
     uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(u_smem_raw) + 1023) & ~(uintptr_t)1023);
     uint64_t* full = reinterpret_cast<uint64_t*>(sm + kUStages * kUStageBytes);
     uint64_t* empty = full + kUStages;
     uint64_t* done = empty + kUStages;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+    uint64_t* sum_full = done + 1;    // a chain of the high parts' products is complete
+    uint64_t* sum_empty = done + 2;   // it has been read
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 3);
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tile0 = blockIdx.x * 4, s = blockIdx.y;
     const int nk = (K + kUKStage - 1) / kUKStage;
     const int k0 = (int)((int64_t)nk * s / S), k1 = (int)((int64_t)nk * (s + 1) / S), ks = k1 - k0;
-    // operand rows of the batch (UMMA N): M rounded up to 16; the rows past M
-    // give accumulator columns that are never read
-    // (the activation parts are stored with this row stride, x3_rows(M))
-    const int N = x3_rows(M);
+    // operand rows of the batch's blocks (UMMA N); the rows of the last one past
+    // M_all give accumulator columns that are never read
+    // (the activation parts are stored with this row stride, x3_rows(M_all))
+    const int N = x3_rows(M_all), row0 = blockIdx.z * N;
+    const int M = M_all - row0 < N ? M_all - row0 : N;  // this block's rows
+    x3 += (int64_t)blockIdx.z * (ldx / 8) * 3 * N * 8;
     const int part_bytes = N * 16;  // one part of one 16-byte chunk
     const uint32_t act_bytes = (uint32_t)(kUKStage / 8 * 3 * part_bytes);
     const uint32_t stage_tx = (uint32_t)kUABytes + act_bytes;
@@ -107,9 +134,11 @@ __global__ void __launch_bounds__(kUThreads, 1)
             u_mb_init(&empty[i], 1);
         }
         u_mb_init(done, 1);
+        u_mb_init(sum_full, 1);
+        u_mb_init(sum_empty, U::EW);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (w == 0) {  // tensor memory for the accumulator
+    if (w == U::EW) {  // tensor memory for the accumulators
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(u_saddr(tmem_slot)),
                      "r"(kUTmemCols)
                      : "memory");
@@ -123,7 +152,7 @@ __global__ void __launch_bounds__(kUThreads, 1)
     // weight blocks are requested before the programmatic wait, so that
     // their HBM latency overlaps the previous kernel's tail.
     const int pre = ks < kUStages ? ks : kUStages;
-    if (w == 0 && lane == 0)
+    if (w == U::EW && lane == 0)
         for (int i = 0; i < pre; ++i) {
             u_expect_tx(&full[i], stage_tx);
             u_tma_w(sm + i * kUStageBytes, &wmap, tile0, (k0 + i) * (kUKStage / 8), &full[i]);
@@ -132,7 +161,7 @@ __global__ void __launch_bounds__(kUThreads, 1)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    if (w == 0 && lane == 0) {
+    if (w == U::EW && lane == 0) {
         // producer: stage i of this split, the ring reused once its MMAs are done
         int issued = 0;
         bool ok = true;
@@ -156,54 +185,124 @@ __global__ void __launch_bounds__(kUThreads, 1)
         // every issued copy lands before the CTA may leave
         for (int i = issued > kUStages ? issued - kUStages : 0; i < issued; ++i)
             u_mb_wait(&full[i % kUStages], (i / kUStages) & 1, nullptr);
-    } else if (w == 1 && lane == 0) {
+    } else if (w == U::EW + 1 && lane == 0) {
         // MMA issuer
         const uint32_t idesc = u_idesc(N);
-        for (int i = 0; i < ks; ++i) {
-            const int st = i % kUStages;
-            if (!u_mb_wait(&full[st], (i / kUStages) & 1, everr)) {
-                atomicOr(err, kErrStall);
-                break;
-            }
+        // each K = 16 step: the weights times the high parts of the block into
+        // the first accumulator, times the middle and the low parts into the
+        // second
+        // (a descriptor's start address is in units of 16 bytes in its low bits)
+        const uint32_t a0 = u_saddr(sm);
+        const uint64_t da0 = u_desc(a0, 2048, 128), db0 = u_desc(a0 + kUABytes, 3 * part_bytes, 128);
+        const uint32_t part16 = part_bytes >> 4;
+        auto mma = [&](int st, int kk, int pp, bool fresh) {
+            const uint32_t at = st * (kUStageBytes >> 4);
+            u_mma(tmem + (pp ? kRowsBlock : 0), da0 + (at + kk * 256), db0 + (at + (kk * 6 + pp) * part16), idesc, fresh ? 0u : 1u);
+        };
+        auto landed = [&](int i) {
+            const bool ok = u_mb_wait(&full[i % kUStages], (i / kUStages) & 1, everr);
+            if (!ok) atomicOr(err, kErrStall);
             u_fence_after();
-            const uint32_t a = u_saddr(sm + st * kUStageBytes), b = a + kUABytes;
-            // each K = 16 step: the weights times the high parts of the batch
-            // into the first accumulator, times the middle and the low parts
-            // into the second
+            return ok;
+        };
+        bool ok = true;
+        for (int i = 0; i < ks && ok;) {
+            if (i > 0 && i % U::CH == 0) {
+                // The high parts start a new chain: two stages' middle and low
+                // parts' products first, which run while the epilogue warps
+                // read the old one.
+                u_commit(sum_full);
+                const int n = ks - i < 2 ? 1 : 2;
+                for (int k = 0; k < n && ok; ++k) {
+                    ok = landed(i + k);
 #pragma unroll
-            for (int kk = 0; kk < kUKStage / 16; ++kk)
+                    for (int kk = 0; kk < kUKStage / 16 && ok; ++kk) {
+                        mma((i + k) % kUStages, kk, 1, false);
+                        mma((i + k) % kUStages, kk, 2, false);
+                    }
+                }
+                if (ok && !u_mb_wait(sum_empty, (i / U::CH - 1) & 1, everr)) {
+                    atomicOr(err, kErrStall);
+                    ok = false;
+                }
+                if (!ok) break;
+                u_fence_after();
+                for (int k = 0; k < n; ++k) {
 #pragma unroll
-                for (int pp = 0; pp < 3; ++pp)
-                    u_mma(tmem + (pp ? kRowsMax : 0), u_desc(a + kk * 2 * 2048, 2048, 128),
-                          u_desc(b + (kk * 2 * 3 + pp) * part_bytes, 3 * part_bytes, 128), idesc,
-                          (i > 0 || kk > 0 || pp == 2) ? 1u : 0u);
-            u_commit(&empty[st]);
+                    for (int kk = 0; kk < kUKStage / 16; ++kk) mma((i + k) % kUStages, kk, 0, k == 0 && kk == 0);
+                    u_commit(&empty[(i + k) % kUStages]);
+                }
+                i += n;
+            } else {
+                ok = landed(i);
+                if (!ok) break;
+#pragma unroll
+                for (int kk = 0; kk < kUKStage / 16; ++kk)
+#pragma unroll
+                    for (int pp = 0; pp < 3; ++pp) mma(i % kUStages, kk, pp, i == 0 && kk == 0 && pp < 2);
+                u_commit(&empty[i % kUStages]);
+                ++i;
+            }
         }
         u_commit(done);  // after every MMA this thread issued
     }
     __syncwarp();
-    // epilogue: every thread is one weight row (tensor-memory lane)
-    bool have = u_mb_wait(done, 0, nullptr);  // the MMA thread commits done after every wait of its own
-    if (!have) have = u_mb_wait(done, 0, nullptr);
-    u_fence_after();
-    // the tensor-memory loads are warp-wide: the whole warp reads or none of it
-    if (__all_sync(0xffffffffu, have && ks > 0 && !(*everr & kErrStall))) {
-        const int n = (tile0 + w) * 32 + lane;  // output row of the projection
-        const uint32_t lane_addr = tmem + ((uint32_t)(32 * w) << 16);
-        float* ps = part + (int64_t)s * M * Np;
-        for (int c0 = 0; c0 < M; c0 += 16) {  // accumulator column = batch row
-            float hi[16], ml[16];
-            u_ld16(lane_addr + c0, hi);
-            u_ld16(lane_addr + kRowsMax + c0, ml);
-            if (tile0 + w < n_tiles)
+    if (w < U::EW) {
+        // epilogue: a thread is one weight row (tensor-memory lane) and half of
+        // the block's rows (accumulator columns)
+        constexpr int HC = U::HC;
+        const int col0 = (w >> 2) * HC, tile = tile0 + (w & 3);
+        const uint32_t lane_addr = tmem + ((uint32_t)(32 * (w & 3)) << 16) + col0;
+        float sum[HC];
 #pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    if (c0 + i < M) ps[(int64_t)(c0 + i) * Np + n] = hi[i] + ml[i];
+        for (int i = 0; i < HC; ++i) sum[i] = 0.f;
+        for (int f = 0; f < (ks - 1) / U::CH; ++f) {
+            if (!u_mb_wait(sum_full, f & 1, everr)) {
+                atomicOr(err, kErrStall);
+                break;
+            }
+            u_fence_after();
+            __syncwarp();
+#pragma unroll
+            for (int c = 0; c < HC; c += 32)
+                if (col0 + c < M) {
+                    uint32_t v0[16], v1[16];
+                    u_ld16(lane_addr + c, v0);
+                    u_ld16(lane_addr + c + 16, v1);
+                    u_wait_ld();
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        sum[c + i] += __uint_as_float(v0[i]);
+                        sum[c + 16 + i] += __uint_as_float(v1[i]);
+                    }
+                }
+            u_fence_before();
+            __syncwarp();
+            if (lane == 0) u_mb_arrive(sum_empty);
+        }
+        bool have = u_mb_wait(done, 0, nullptr);  // the MMA thread commits done after every wait of its own
+        if (!have) have = u_mb_wait(done, 0, nullptr);
+        u_fence_after();
+        // the tensor-memory loads are warp-wide: the whole warp reads or none of it
+        if (__all_sync(0xffffffffu, have && ks > 0 && !(*everr & kErrStall))) {
+            const int n = tile * 32 + lane;  // output row of the projection
+            float* ps = part + ((int64_t)s * M_all + row0 + col0) * Np;
+#pragma unroll
+            for (int c = 0; c < HC; c += 16)
+                if (col0 + c < M) {
+                    float hi[16], ml[16];
+                    u_ld16(lane_addr + c, hi);
+                    u_ld16(lane_addr + kRowsBlock + c, ml);
+                    if (tile < n_tiles)
+#pragma unroll
+                        for (int i = 0; i < 16; ++i)
+                            if (col0 + c + i < M) ps[(int64_t)(c + i) * Np + n] = sum[c + i] + (hi[i] + ml[i]);
+                }
         }
     }
     u_fence_before();
     __syncthreads();
-    if (w == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kUTmemCols) : "memory");
+    if (w == U::EW) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kUTmemCols) : "memory");
 }
 
 // ---------------------------------------------------------------- host side
@@ -253,7 +352,9 @@ bool umma_available() {
         CUtensorMap probe;
         static uint16_t dummy[64 * 8] __attribute__((aligned(16)));
         ok = major == 10 && encode_fn() && weight_map(&probe, dummy, 4, 64) &&
-             cudaFuncSetAttribute(k_rows_umma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)umma_smem()) ==
+             cudaFuncSetAttribute(k_rows_umma<ULarge>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)umma_smem()) ==
+                 cudaSuccess &&
+             cudaFuncSetAttribute(k_rows_umma<USmall>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)umma_smem()) ==
                  cudaSuccess &&
              configure_uattn() == cudaSuccess;
         cudaGetLastError();
@@ -263,22 +364,23 @@ bool umma_available() {
 
 // K splits: as many as keep the grid within one wave (one CTA per SM: the
 // stages take most of the shared memory), at most one per stage.
-int umma_splits(int64_t n_tiles, int K, int n_sm) {
-    const int64_t mt = (n_tiles + 3) / 4;
+int umma_splits(int64_t n_tiles, int K, int M, int n_sm) {
+    const int64_t mt = (n_tiles + 3) / 4 * rows_blocks(M);
     const int nk = (K + kUKStage - 1) / kUKStage;
     const int64_t want = n_sm / mt;
     return (int)std::max<int64_t>(1, std::min<int64_t>(want, nk));
 }
 
-cudaError_t launch_mm_umma(const uint16_t* W, int64_t n_rows, int K, const uint16_t* x3, int M, int S, float* part,
+cudaError_t launch_mm_umma(const uint16_t* W, int64_t n_rows, int K, const uint16_t* x3, int ldx, int M, int S, float* part,
                            int Np, int* err, cudaStream_t s) {
     const int64_t nt = tile_count(n_rows);
     CUtensorMap map;
     if (!weight_map(&map, W, nt, K)) return cudaErrorNotSupported;
-    const dim3 grid((unsigned)((nt + 3) / 4), (unsigned)S);
+    const dim3 grid((unsigned)((nt + 3) / 4), (unsigned)S, (unsigned)rows_blocks(M));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
-    cfg.blockDim = dim3(kUThreads);
+    const bool small = x3_rows(M) <= USmall::EW / 4 * USmall::HC;
+    cfg.blockDim = dim3(small ? USmall::threads : ULarge::threads);
     cfg.dynamicSmemBytes = umma_smem();
     cfg.stream = s;
     cudaLaunchAttribute at[1];
@@ -286,7 +388,8 @@ cudaError_t launch_mm_umma(const uint16_t* W, int64_t n_rows, int K, const uint1
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_rows_umma, map, x3, (int)nt, K, M, S, part, Np, err);
+    if (small) return cudaLaunchKernelEx(&cfg, k_rows_umma<USmall>, map, x3, ldx, (int)nt, K, M, S, part, Np, err);
+    return cudaLaunchKernelEx(&cfg, k_rows_umma<ULarge>, map, x3, ldx, (int)nt, K, M, S, part, Np, err);
 }
 
 }  // namespace ee

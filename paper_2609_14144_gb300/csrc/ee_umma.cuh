@@ -39,6 +39,10 @@ __device__ __forceinline__ bool u_mb_wait(uint64_t* b, int parity, const volatil
     }
 }
 
+__device__ __forceinline__ void u_mb_arrive(uint64_t* b) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(u_saddr(b)) : "memory");
+}
+
 // ---------------------------------------------------------------- tcgen05
 // Shared-memory operand descriptor, no swizzle: start address and the byte
 // offsets between core matrices (8 x 16 bytes, contiguous) along K (lbo) and

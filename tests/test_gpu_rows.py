@@ -111,12 +111,14 @@ def test_tiny_prompt_paths_agree(tiny_model):
 
 
 @pytest.mark.parametrize("D,page", [(64, 16), (64, 256), (128, 64), (128, 32)])
-@pytest.mark.parametrize("n", [64, 65, 127, 129, 193, 700])
+@pytest.mark.parametrize("n", [64, 65, 127, 129, 193, 513, 1025])
 def test_tcgen05_attention_row_and_key_edges(n, D, page):
     """The batched attention at the edges of its row tile (128 rows, from 65
     on), of a block of 64 keys and of a key split, with pages shorter and
-    longer than a block in any order, seven query heads to a key-value head:
-    against the same prompt one position at a time (fp32 path)."""
+    longer than a block in any order, seven query heads to a key-value head;
+    the batch at the edges of the products' row blocks (256 rows; 513 makes
+    three of 176) and of its own size (1025 makes two batches): against the
+    same prompt one position at a time (fp32 path)."""
     from paper_2609_14144_gb300 import OPT_DEBUG_LOGITS, OPT_ROWS, Engine
 
     shape = TINY.replace(n_heads=14, head_dim=D, n_layers=2, readout_layers=(1,))
