@@ -261,12 +261,15 @@ __host__ __device__ constexpr int x3_rows(int M) {
     return ((M + rows_blocks(M) - 1) / rows_blocks(M) + 15) & ~15;
 }
 constexpr int kRowsTargetUnits = 2432;   // (tile, K split) units a projection aims for: 152 SMs x 16 warps
+// Floats a row and head of one attention split takes: D unnormalised outputs,
+// maximum, sum, and two so that every one starts on 16 bytes.
+__host__ __device__ constexpr int kAttnLd(int D) { return D + 4; }
 struct RowsBuf {
     float* H;           // [kRowsMax][d] residual of each row
     uint16_t* x3;       // next product's input as three bf16 parts (high, x - high, the rest),
                         // chunk-major: [blocks][ldx / 8][3][x3_rows(M)][8] for a batch of M rows
     float* Q;           // [kRowsMax][A D] rotated queries
-    float* part;        // split partials [S][M][n_rows padded to 32] of a projection, [S][M][A][D + 2] of the attention
+    float* part;        // split partials [S][M][n_rows padded to 32] of a projection, [S][M][A][kAttnLd(D)] of the attention
     int32_t* pos;       // [kRowsMax] positions of a prompt batch
     int64_t part_floats;
     int ldx;

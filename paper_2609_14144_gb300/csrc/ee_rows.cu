@@ -71,16 +71,35 @@ struct Parts {
     }
 };
 
-// The three bf16 parts of x at (row, col): high = bf16(x), middle = bf16(x -
-// high), low = bf16(x - high - middle) (each difference exact in fp32).
-__device__ __forceinline__ void split_store(float x, const Parts& p, int row, int col) {
-    const uint16_t h = r_f2bf(x);
-    const float r1 = x - r_bf2f(h);
-    const uint16_t md = r_f2bf(r1);
-    const int64_t at = p.index(0, row, col);
-    p.p[at] = h;
-    p.p[at + p.rows * 8] = md;
-    p.p[at + p.rows * 16] = r_f2bf(r1 - r_bf2f(md));
+// Two values as three packed bf16 parts: high = bf16(x), middle = bf16(x -
+// high), low = bf16(x - high - middle) (each difference exact in fp32); four
+// columns of a row stored from `at` on (its high part), and eight (a whole
+// chunk), one store per part.
+__device__ __forceinline__ void split_pair(float a, float b, uint32_t (&p)[3]) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);  // a in the low half
+        p[k] = *reinterpret_cast<const uint32_t*>(&v);
+        a -= __uint_as_float(p[k] << 16);
+        b -= __uint_as_float(p[k] & 0xffff0000u);
+    }
+}
+__device__ __forceinline__ void split_store4(float4 x, const Parts& p, int64_t at) {
+    uint32_t a[3], b[3];
+    split_pair(x.x, x.y, a);
+    split_pair(x.z, x.w, b);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) *reinterpret_cast<uint2*>(p.p + at + k * p.rows * 8) = make_uint2(a[k], b[k]);
+}
+__device__ __forceinline__ void split_store8(const float (&x)[8], const Parts& p, int64_t at) {
+    uint32_t a[3], b[3], c[3], d[3];
+    split_pair(x[0], x[1], a);
+    split_pair(x[2], x[3], b);
+    split_pair(x[4], x[5], c);
+    split_pair(x[6], x[7], d);
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        *reinterpret_cast<uint4*>(p.p + at + k * p.rows * 8) = make_uint4(a[k], b[k], c[k], d[k]);
 }
 // Columns from n up to the next multiple of 64 (a tensor-core stage) read as 0.
 __host__ __device__ __forceinline__ int pad64(int n) { return (n + 63) & ~63; }
@@ -219,63 +238,100 @@ __global__ void __launch_bounds__(kRowsThreads) k_rows_mm(const uint4* __restric
 
 // ------------------------------------------------------------------ per-row epilogues
 
-constexpr int kNormThreads = 768;  // residual add + RMSNorm: one CTA per row
-
-// Sum over the block of NT threads; every thread gets the same value (fixed order).
-template <int NT>
+// Sum over the block (of at most 1024 threads); every thread gets the same
+// value (fixed order).
 __device__ __forceinline__ float r_block_sum(float v, float* red) {
     v = r_warp_sum(v);
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
     __syncthreads();
     if (l == 0) red[w] = v;
     __syncthreads();
-    float t = l < NT / 32 ? red[l] : 0.f;
+    float t = l < (int)(blockDim.x >> 5) ? red[l] : 0.f;
     return r_warp_sum(t);
 }
 
-// Sum of the S split partials p[0], p[stride], ..., in a fixed order: four
-// running sums over splits s = 4k + r, added pairwise at the end, so that
-// several loads are in flight.
-__device__ __forceinline__ float split_sum(const float* __restrict__ p, int64_t stride, int S) {
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+__device__ __forceinline__ float2 radd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float4 radd(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+template <class T>
+__device__ __forceinline__ T rzero();
+template <>
+__device__ __forceinline__ float2 rzero<float2>() { return make_float2(0.f, 0.f); }
+template <>
+__device__ __forceinline__ float4 rzero<float4>() { return make_float4(0.f, 0.f, 0.f, 0.f); }
+
+// Sum of the S split partials p[0], p[stride], ... (T: two or four
+// neighbouring columns), in a fixed order: four running sums over splits s = 4k
+// + r, added pairwise at the end, so that several loads are in flight.
+template <class T>
+__device__ __forceinline__ T split_sum(const float* __restrict__ p, int64_t stride, int S) {
+    auto at = [&](int s) { return *reinterpret_cast<const T*>(p + (int64_t)s * stride); };
+    T a0 = rzero<T>(), a1 = a0, a2 = a0, a3 = a0;
     int s = 0;
 #pragma unroll 2
     for (; s + 4 <= S; s += 4) {
-        a0 += p[(int64_t)s * stride];
-        a1 += p[(int64_t)(s + 1) * stride];
-        a2 += p[(int64_t)(s + 2) * stride];
-        a3 += p[(int64_t)(s + 3) * stride];
+        const T v0 = at(s), v1 = at(s + 1), v2 = at(s + 2), v3 = at(s + 3);
+        a0 = radd(a0, v0);
+        a1 = radd(a1, v1);
+        a2 = radd(a2, v2);
+        a3 = radd(a3, v3);
     }
-    for (; s < S; ++s) a0 += p[(int64_t)s * stride];
-    return (a0 + a1) + (a2 + a3);
+#pragma unroll 1
+    for (; s < S; ++s) a0 = radd(a0, at(s));
+    return radd(radd(a0, a1), radd(a2, a3));
 }
 
-// One CTA per row i < M_norm.  Rows below M_add first add the split partials
-// of a d-output projection (split stride M_add rows) to their residual.  With
-// a gain, the row's RMSNorm h / sqrt(mean(h^2) + eps) * g goes to x as three
-// bf16 parts.
-__global__ void __launch_bounds__(kNormThreads) k_rows_add_norm(float* __restrict__ H, int d,
+// One CTA per row i < M_norm, a thread takes four neighbouring columns (four
+// more 4 blockDim further on, for rows longer than that).  Rows below M_add
+// first add the split partials of a d-output projection (split stride M_add
+// rows) to their residual.  With a gain, the row's RMSNorm
+// h / sqrt(mean(h^2) + eps) * g goes to x as three bf16 parts.
+// The launch is a chain of latencies (partials, block sum, store), so a row is
+// spread over as many threads as it has groups of four columns, every load is
+// 16 bytes and in flight with the others, and what a thread holds of a row of up
+// to 4096 columns stays in registers between the two halves.
+constexpr int kNormMaxThreads = 1024;
+__host__ __device__ constexpr int norm_threads(int d) {
+    return d / 4 >= kNormMaxThreads ? kNormMaxThreads : (d / 4 + 31) / 32 * 32;
+}
+__global__ void __launch_bounds__(kNormMaxThreads) k_rows_add_norm(float* __restrict__ H, int d,
                                                                 const float* __restrict__ part, int S, int M_add,
                                                                 int Np, const uint16_t* __restrict__ gain, float eps,
-                                                                const Parts x3, int ldx) {
+                                                                const Parts x3) {
+    __shared__ float red[kNormMaxThreads / 32];
+    const int i = blockIdx.x, n0 = 4 * threadIdx.x, step = 4 * blockDim.x;
+    // (the gain does not depend on the launch before)
+    const uint2 g0 = gain && n0 < d ? __ldg(reinterpret_cast<const uint2*>(gain + n0)) : make_uint2(0u, 0u);
     r_pdl();
-    __shared__ float red[kNormThreads / 32];
-    const int i = blockIdx.x;
     float* h = H + (int64_t)i * d;
     float ss = 0.f;
-    for (int n = threadIdx.x; n < d; n += kNormThreads) {
-        float v = h[n];
+    float4 v0 = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+    for (int n = n0; n < d; n += step) {
+        float4 v = *reinterpret_cast<const float4*>(h + n);
         if (i < M_add) {
-            v += split_sum(part + (int64_t)i * Np + n, (int64_t)M_add * Np, S);
-            h[n] = v;
+            v = radd(v, split_sum<float4>(part + (int64_t)i * Np + n, (int64_t)M_add * Np, S));
+            *reinterpret_cast<float4*>(h + n) = v;
         }
-        ss = fmaf(v, v, ss);
+        ss = fmaf(v.x, v.x, ss);
+        ss = fmaf(v.y, v.y, ss);
+        ss = fmaf(v.z, v.z, ss);
+        ss = fmaf(v.w, v.w, ss);
+        if (n == n0) v0 = v;
     }
     if (!gain) return;  // uniform over the block
-    ss = r_block_sum<kNormThreads>(ss, red);
+    ss = r_block_sum(ss, red);
     const float inv = 1.0f / sqrtf(ss / (float)d + eps);
-    for (int n = threadIdx.x; n < pad64(d); n += kNormThreads)
-        split_store(n < d ? h[n] * inv * r_bf2f(gain[n]) : 0.f, x3, i, n);
+#pragma unroll 1
+    for (int n = n0; n < pad64(d); n += step) {
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (n < d) {
+            const float4 v = n == n0 ? v0 : *reinterpret_cast<const float4*>(h + n);
+            const uint2 g = n == n0 ? g0 : __ldg(reinterpret_cast<const uint2*>(gain + n));
+            x = make_float4(v.x * inv * __uint_as_float(g.x << 16), v.y * inv * __uint_as_float(g.x & 0xffff0000u),
+                            v.z * inv * __uint_as_float(g.y << 16), v.w * inv * __uint_as_float(g.y & 0xffff0000u));
+        }
+        split_store4(x, x3, x3.index(0, i, n));
+    }
 }
 
 // Q/K/V of layer j for row blockIdx.y: thread = one unit (the packed row pair
@@ -290,8 +346,8 @@ __global__ void __launch_bounds__(kRowsThreads) k_rows_qkv(DevModel m, int j, co
     const int half = m.D >> 1;
     const int nq = m.A * half, nk = m.KH * half;
     if (u >= nq + 2 * nk) return;
-    const float* p = part + (int64_t)i * Np + 2 * u;
-    float r0 = split_sum(p, (int64_t)M * Np, S), r1 = split_sum(p + 1, (int64_t)M * Np, S);
+    const float2 rr = split_sum<float2>(part + (int64_t)i * Np + 2 * u, (int64_t)M * Np, S);
+    float r0 = rr.x, r1 = rr.y;
     if (m.qkv_bias) {
         const uint16_t* b = m.layers + (int64_t)j * m.layer_stride + m.off_bqkv;
         r0 += r_bf2f(b[2 * u]);
@@ -319,22 +375,32 @@ __global__ void __launch_bounds__(kRowsThreads) k_rows_qkv(DevModel m, int j, co
     if (u == 0) m.kv_src[(int64_t)j * m.max_ctx + t] = 1;
 }
 
-// SwiGLU of row blockIdx.y: a = silu(gate) * up from the split sums of the
-// packed (gate, up) row pair, as three bf16 parts.
+// SwiGLU: a = silu(gate) * up from the split sums of the packed (gate, up) row
+// pairs, as three bf16 parts.  A thread takes eight features (one 16-byte chunk)
+// of one row, a warp four chunks of eight rows: it reads 256 contiguous bytes a
+// row and split and writes 128 contiguous bytes a chunk and part.
+constexpr int kSwigluRows = 8, kSwigluChunks = kRowsThreads / kSwigluRows;
 __global__ void __launch_bounds__(kRowsThreads) k_rows_swiglu(const float* __restrict__ part, int S, int M, int Np,
-                                                              int F, const Parts x3, int ldx) {
+                                                              int F, const Parts x3) {
     r_pdl();
-    const int i = blockIdx.y;
-    const int f = blockIdx.x * kRowsThreads + threadIdx.x;
-    if (f >= pad64(F)) return;
-    if (f >= F) {
-        split_store(0.f, x3, i, f);
-        return;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int i = blockIdx.y * kSwigluRows + (lane >> 2), c = blockIdx.x * kSwigluChunks + w * 4 + (lane & 3);
+    if (i >= M || 8 * c >= pad64(F)) return;
+    float x[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) x[e] = 0.f;
+    if (8 * c < F) {  // (F is a multiple of 8)
+        const float* p = part + (int64_t)i * Np + 16 * c;
+        float4 v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = split_sum<float4>(p + 4 * q, (int64_t)M * Np, S);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            x[2 * q] = v[q].x / (1.0f + expf(-v[q].x)) * v[q].y;
+            x[2 * q + 1] = v[q].z / (1.0f + expf(-v[q].z)) * v[q].w;
+        }
     }
-    const float* p = part + (int64_t)i * Np + 2 * f;
-    const float gs = split_sum(p, (int64_t)M * Np, S), us = split_sum(p + 1, (int64_t)M * Np, S);
-    const float a = gs / (1.0f + expf(-gs)) * us;
-    split_store(a, x3, i, f);
+    split_store8(x, x3, x3.index(0, i, 8 * c));
 }
 
 // Starting residual of row blockIdx.x: the embedding of ids[i] (a prompt;
@@ -603,8 +669,8 @@ __global__ void __launch_bounds__(kFaThreads) k_rows_fattn(DevModel m, int j, co
     }
     if (!act) return;
     // the split's unnormalised output, maximum and sum of each row:
-    // part[((s Mj + row) A + h)][D + 2]
-    const int ld = D + 2;
+    // part[((s Mj + row) A + h)][kAttnLd(D)]
+    constexpr int ld = kAttnLd(D);
     float* q0 = part + ((int64_t)(s * Mj + r0) * m.A + h) * ld;
     float* q1 = part + ((int64_t)(s * Mj + r1) * m.A + h) * ld;
 #pragma unroll
@@ -631,30 +697,39 @@ __global__ void __launch_bounds__(kFaThreads) k_rows_fattn(DevModel m, int j, co
     }
 }
 
-// The splits of row i, head h (blockIdx.x = h, blockIdx.y = i; D threads):
-// o = sum_s exp(m_s - M) o_s / sum_s exp(m_s - M) l_s over the splits that
-// hold a key at or before the row's position, in split order; written as the
-// O projection's three bf16 parts at column h D + e.
+// The splits of a row and head: o = sum_s exp(m_s - M) o_s / sum_s exp(m_s - M)
+// l_s over the splits that hold a key at or before the row's position, in split
+// order; written as the O projection's three bf16 parts at column h D + e.
+// blockIdx.x = h; D / 4 threads a row, each four dimensions, eight rows a CTA.
+constexpr int kMergeRows = 8;
 template <int D>
-__global__ void __launch_bounds__(D) k_rows_amerge(DevModel m, const float* __restrict__ part,
-                                                   const int32_t* __restrict__ pos, int KC, const Parts x3) {
+__global__ void __launch_bounds__(kMergeRows * D / 4) k_rows_amerge(DevModel m, const float* __restrict__ part, int Mj,
+                                                     const int32_t* __restrict__ pos, int KC, const Parts x3) {
     r_pdl();
-    const int h = blockIdx.x, i = blockIdx.y, e = threadIdx.x;
-    const int ns = pos[i] / KC + 1, ld = D + 2;
+    const int h = blockIdx.x, i = blockIdx.y * kMergeRows + threadIdx.x / (D / 4), e = 4 * (threadIdx.x % (D / 4));
+    if (i >= Mj) return;
+    constexpr int ld = kAttnLd(D);
+    const int ns = pos[i] / KC + 1;
     const float* q = part + ((int64_t)i * m.A + h) * ld;
-    const int64_t step = (int64_t)gridDim.y * m.A * ld;  // one split
+    const int64_t step = (int64_t)Mj * m.A * ld;  // one split
     float M = -INFINITY;
     for (int s = 0; s < ns; ++s) M = fmaxf(M, q[s * step + D]);
-    float num = 0.f, den = 0.f;
+    float4 num = make_float4(0.f, 0.f, 0.f, 0.f);
+    float den = 0.f;
     for (int s = 0; s < ns; ++s) {
         const float* qs = q + s * step;
         const float wgt = expf(qs[D] - M);
-        num = fmaf(wgt, qs[e], num);
+        const float4 o = *reinterpret_cast<const float4*>(qs + e);
+        num.x = fmaf(wgt, o.x, num.x);
+        num.y = fmaf(wgt, o.y, num.y);
+        num.z = fmaf(wgt, o.z, num.z);
+        num.w = fmaf(wgt, o.w, num.w);
         den = fmaf(wgt, qs[D + 1], den);
     }
-    split_store(num / den, x3, i, h * D + e);
+    split_store4(make_float4(num.x / den, num.y / den, num.z / den, num.w / den), x3, x3.index(0, i, h * D + e));
     if (h == 0)  // the columns past A D up to the tensor cores' stage
-        for (int col = m.A * D + e; col < pad64(m.A * D); col += D) split_store(0.f, x3, i, col);
+        for (int col = m.A * D + e; col < pad64(m.A * D); col += D)
+            split_store4(make_float4(0.f, 0.f, 0.f, 0.f), x3, x3.index(0, i, col));
 }
 
 // ------------------------------------------------------------------ host side
@@ -708,6 +783,12 @@ int fa_keys_per_split(int t_max, int units, int n_sm, int max_splits) {
 // kFaMaxSplits splits of kRowsBlock rows take.
 int attn_splits(int M) { return std::max(1, std::min(kFaMaxSplits, kFaMaxSplits * kRowsBlock / M)); }
 
+template <int D>
+cudaError_t launch_merge(const DevModel& m, const RowsBuf& b, int Mj, const int32_t* d_pos, int KC, cudaStream_t s) {
+    return launch_pdl(k_rows_amerge<D>, dim3(m.A, (Mj + kMergeRows - 1) / kMergeRows), dim3(kMergeRows * D / 4), 0, s, m,
+                      (const float*)b.part, Mj, d_pos, KC, parts(b, Mj));
+}
+
 // The batch's attention at layer j: the split kernel, then the merge into
 // the O projection's input parts.
 cudaError_t launch_attn(const DevModel& m, const RowsBuf& b, int j, int Mj, const int32_t* d_pos, int t_max,
@@ -716,9 +797,8 @@ cudaError_t launch_attn(const DevModel& m, const RowsBuf& b, int j, int Mj, cons
         const int KC = uattn_keys_per_split(t_max, m.A, Mj, b.n_sm, attn_splits(Mj));
         RCKA(launch_uattn(m, j, b.Q, d_pos, Mj, KC, t_max, b.part, s));
         if (m.D == 128)
-            return launch_pdl(k_rows_amerge<128>, dim3(m.A, Mj), dim3(128), 0, s, m, (const float*)b.part, d_pos, KC,
-                              parts(b, Mj));
-        return launch_pdl(k_rows_amerge<64>, dim3(m.A, Mj), dim3(64), 0, s, m, (const float*)b.part, d_pos, KC, parts(b, Mj));
+            return launch_merge<128>(m, b, Mj, d_pos, KC, s);
+        return launch_merge<64>(m, b, Mj, d_pos, KC, s);
     }
     const int row_blocks = (Mj + kFaWarps * 16 - 1) / (kFaWarps * 16);
     const int KC = fa_keys_per_split(t_max, m.A * row_blocks, b.n_sm, attn_splits(Mj));
@@ -727,12 +807,11 @@ cudaError_t launch_attn(const DevModel& m, const RowsBuf& b, int j, int Mj, cons
     if (m.D == 128) {
         RCKA(launch_pdl(k_rows_fattn<128>, grid, dim3(kFaThreads), fa_smem(128), s, m, j, (const float*)b.Q, d_pos, Mj,
                         KC, t_max, b.part));
-        return launch_pdl(k_rows_amerge<128>, dim3(m.A, Mj), dim3(128), 0, s, m, (const float*)b.part, d_pos, KC,
-                          parts(b, Mj));
+        return launch_merge<128>(m, b, Mj, d_pos, KC, s);
     }
     RCKA(launch_pdl(k_rows_fattn<64>, grid, dim3(kFaThreads), fa_smem(64), s, m, j, (const float*)b.Q, d_pos, Mj, KC,
                     t_max, b.part));
-    return launch_pdl(k_rows_amerge<64>, dim3(m.A, Mj), dim3(64), 0, s, m, (const float*)b.part, d_pos, KC, parts(b, Mj));
+    return launch_merge<64>(m, b, Mj, d_pos, KC, s);
 }
 
 // One projection of the batch: W (n_rows x K, tiled) times the M rows of
@@ -802,8 +881,8 @@ int64_t rows_part_floats(int d, int A, int KH, int D, int F) {
             const int64_t nt = tile_count(rows[p]);
             most = std::max(most, (int64_t)rows_splits(nt, K[p], M) * M * nt * kTileRows);
         }
-    // the attention's split outputs: [attn_splits(M)][M][A][D + 2]
-    return std::max(most, (int64_t)kFaMaxSplits * kRowsBlock * A * (D + 2));
+    // the attention's split outputs: [attn_splits(M)][M][A][kAttnLd(D)]
+    return std::max(most, (int64_t)kFaMaxSplits * kRowsBlock * A * kAttnLd(D));
 }
 
 #define RCK(x)                                    \
@@ -831,8 +910,8 @@ cudaError_t rows_pass(const DevModel& m, const RowsBuf& b_in, const int* start, 
         const uint16_t* lw = m.layers + (int64_t)j * m.layer_stride;
         int S = 1, Np = 0;
         // the previous layer's down projection into the residual, this layer's input norm
-        RCK(launch_pdl(k_rows_add_norm, dim3(Mj), dim3(kNormThreads), 0, s, b.H, d, (const float*)b.part, S_prev, M_prev,
-                       Np_prev, lw + m.off_gattn, m.eps, parts(b, Mj), b.ldx));
+        RCK(launch_pdl(k_rows_add_norm, dim3(Mj), dim3(norm_threads(d)), 0, s, b.H, d, (const float*)b.part, S_prev, M_prev,
+                       Np_prev, lw + m.off_gattn, m.eps, parts(b, Mj)));
         RCK(launch_mm(lw + m.off_wqkv, nqkv, d, b, Mj, S, Np, s));
         const int nu = (int)(nqkv / 2);
         RCK(launch_pdl(k_rows_qkv, dim3((nu + kRowsThreads - 1) / kRowsThreads, Mj), dim3(kRowsThreads), 0, s, m, j,
@@ -848,19 +927,20 @@ cudaError_t rows_pass(const DevModel& m, const RowsBuf& b_in, const int* start, 
         }
         RCK(launch_attn(m, b, j, Mj, d_pos, t_max, s));
         RCK(launch_mm(lw + m.off_wo, d, AD, b, Mj, S, Np, s));
-        RCK(launch_pdl(k_rows_add_norm, dim3(Mj), dim3(kNormThreads), 0, s, b.H, d, (const float*)b.part, S, Mj, Np,
-                       lw + m.off_gmlp, m.eps, parts(b, Mj), b.ldx));
+        RCK(launch_pdl(k_rows_add_norm, dim3(Mj), dim3(norm_threads(d)), 0, s, b.H, d, (const float*)b.part, S, Mj, Np,
+                       lw + m.off_gmlp, m.eps, parts(b, Mj)));
         RCK(launch_mm(lw + m.off_wgu, 2LL * m.F, d, b, Mj, S, Np, s));
-        RCK(launch_pdl(k_rows_swiglu, dim3((pad64(m.F) + kRowsThreads - 1) / kRowsThreads, Mj), dim3(kRowsThreads), 0, s,
-                       (const float*)b.part, S, Mj, Np, m.F, parts(b, Mj), b.ldx));
+        RCK(launch_pdl(k_rows_swiglu, dim3((pad64(m.F) / 8 + kSwigluChunks - 1) / kSwigluChunks,
+                                           (Mj + kSwigluRows - 1) / kSwigluRows), dim3(kRowsThreads), 0, s,
+                       (const float*)b.part, S, Mj, Np, m.F, parts(b, Mj)));
         RCK(launch_mm(lw + m.off_wd, d, m.F, b, Mj, S, Np, s));
         M_prev = Mj;
         S_prev = S;
         Np_prev = Np;
     }
     // the last down projection into the residual (no norm)
-    return launch_pdl(k_rows_add_norm, dim3(M_prev), dim3(kNormThreads), 0, s, b.H, d, (const float*)b.part, S_prev,
-                      M_prev, Np_prev, (const uint16_t*)nullptr, m.eps, parts(b, M_prev), b.ldx);
+    return launch_pdl(k_rows_add_norm, dim3(M_prev), dim3(norm_threads(d)), 0, s, b.H, d, (const float*)b.part, S_prev,
+                      M_prev, Np_prev, (const uint16_t*)nullptr, m.eps, parts(b, M_prev));
 }
 
 cudaError_t launch_rows_prefill_done(const DevModel& m, int n, cudaStream_t s) {

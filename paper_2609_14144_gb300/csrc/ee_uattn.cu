@@ -327,14 +327,15 @@ __global__ void __launch_bounds__(kUaThreads, 1)
         if (*everr & kErrStall) u_mb_wait(pv_done, (nb - 1) & 1, nullptr);  // products in flight end
         add_products();
         ua_wait_group<0>();
-        // the split's unnormalised output, maximum and sum: part[((s Mj + row) A + h)][D + 2]
+        // the split's unnormalised output, maximum and sum: part[((s Mj + row) A + h)][kAttnLd(D)]
         __syncthreads();
         xch[qt * kUaRows + row] = l;
         __syncthreads();
         if (my_pos >= k0) {
-            float* out = part + ((int64_t)(s * Mj + r0 + row) * m.A + h) * (D + 2);
+            float* out = part + ((int64_t)(s * Mj + r0 + row) * m.A + h) * kAttnLd(D);
 #pragma unroll
-            for (int i = 0; i < HC; i += 2) *reinterpret_cast<float2*>(out + qt * HC + i) = make_float2(o[i], o[i + 1]);
+            for (int i = 0; i < HC; i += 4)
+                *reinterpret_cast<float4*>(out + qt * HC + i) = make_float4(o[i], o[i + 1], o[i + 2], o[i + 3]);
             float lt = 0.f;
 #pragma unroll
             for (int e = 0; e < kUaSplit; ++e) lt += xch[e * kUaRows + row];
