@@ -52,7 +52,7 @@ namespace {
 constexpr int kCW = kSegConsumerWarps;
 constexpr int kCT = 32 * kCW;              // consumer threads
 constexpr int kColsPerChunk = kSegChunk / (2 * kTileRows);  // 512
-constexpr int kCCPerWarp = (kColsPerChunk / 8 + kCW - 1) / kCW;  // 16-byte column chunks a warp takes per stage
+constexpr int kRedSlots = 4;               // tiles whose partial row sums wait for one meeting of the warps (at most)
 // Wait bounds are in SM clock cycles (kSegStallCycles, kSegCheckCycles;
 // clock64 is cheap to read, the error word in global memory is not, so a
 // waiting thread looks at it only once per check interval).
@@ -246,42 +246,74 @@ __device__ __forceinline__ float dot8s(const uint4 w, uint32_t xa) {
     s = fmaf(bfhi(w.w), b.w, s);
     return s;
 }
-// Dot products of one ring stage for one warp: lane = row of the tile, the
-// warp's 16-byte column chunks are w, w + kCW, ... (stage byte address `wl`
-// already offset by lane * 16 + w * 512, input address `xl` by w * 32).
-// Full stages take the branch-free path with every chunk's product an
-// independent chain; a ragged last stage of a row checks each chunk.
-template <int CC>
-__device__ __forceinline__ float stage_dot(uint32_t wl, uint32_t xl, int cc_first, int ccn) {
-    if (cc_first + (CC - 1) * kSegConsumerWarps < ccn) {
-        uint4 wv[CC];
+// Running dot products of one warp over ring stages: lane (c4, r8) = (lane /
+// 8, lane mod 8) holds the sums of rows r8, r8 + 8, r8 + 16 and r8 + 24 of
+// the tile over its own 16-byte column chunks, even and odd columns apart.
+// The four rows share each load of the input (one row per lane takes two
+// input loads for every weight load, and a 16-byte load costs the
+// shared-memory pipe four cycles, broadcast or not); eight rows would make
+// the eight lanes of a load phase read from two column chunks, 512 bytes
+// apart: the same banks.
+struct RowAcc {
+    float2 a[4];
+    __device__ __forceinline__ void clear() {
 #pragma unroll
-        for (int u = 0; u < CC; ++u) wv[u] = lds128(wl + u * kSegConsumerWarps * 512);
-        float a[CC];
-#pragma unroll
-        for (int u = 0; u < CC; ++u) {
-            const float4 x0 = lds128f(xl + u * kSegConsumerWarps * 32);
-            const float4 x1 = lds128f(xl + u * kSegConsumerWarps * 32 + 16);
-            float p0 = bflo(wv[u].x) * x0.x, p1 = bfhi(wv[u].x) * x0.y;
-            p0 = fmaf(bflo(wv[u].y), x0.z, p0);
-            p1 = fmaf(bfhi(wv[u].y), x0.w, p1);
-            p0 = fmaf(bflo(wv[u].z), x1.x, p0);
-            p1 = fmaf(bfhi(wv[u].z), x1.y, p1);
-            p0 = fmaf(bflo(wv[u].w), x1.z, p0);
-            p1 = fmaf(bfhi(wv[u].w), x1.w, p1);
-            a[u] = p0 + p1;
-        }
-        float t = 0.f;
-#pragma unroll
-        for (int u = 0; u < CC; ++u) t += a[u];
-        return t;
+        for (int q = 0; q < 4; ++q) a[q] = make_float2(0.f, 0.f);
     }
-    float t = 0.f;
-    for (int u = 0; cc_first + u * kSegConsumerWarps < ccn; ++u)
-        t += dot8s(lds128(wl + u * kSegConsumerWarps * 512), xl + u * kSegConsumerWarps * 32);
-    return t;
+    // The warp's total of row `lane` of the tile: a transposing sum over the
+    // four column groups (rows r8 + 8 c4 end on lane (c4, r8)).
+    __device__ __forceinline__ float total() const {
+        const int lane = threadIdx.x & 31;
+        const bool hi = lane & 16, odd = lane & 8;
+        const float s0 = a[0].x + a[0].y, s1 = a[1].x + a[1].y, s2 = a[2].x + a[2].y, s3 = a[3].x + a[3].y;
+        float k0 = hi ? s2 : s0, k1 = hi ? s3 : s1;
+        k0 += __shfl_xor_sync(0xffffffffu, hi ? s0 : s2, 16);
+        k1 += __shfl_xor_sync(0xffffffffu, hi ? s1 : s3, 16);
+        return (odd ? k1 : k0) + __shfl_xor_sync(0xffffffffu, odd ? k0 : k1, 8);
+    }
+};
+// This lane's first column chunk of a stage; its byte offset in the stage's
+// weights and in the input columns.
+constexpr int kStageStep = 4 * kSegConsumerWarps;        // column chunks the CTA takes at once
+constexpr int kStageU = kColsPerChunk / 8 / kStageStep;  // column chunks a lane takes of a full stage
+__device__ __forceinline__ int stage_c0() { return (threadIdx.x >> 5) * 4 + ((threadIdx.x & 31) >> 3); }
+__device__ __forceinline__ uint32_t stage_woff() { return stage_c0() * 512 + (threadIdx.x & 7) * 16; }
+__device__ __forceinline__ uint32_t stage_xoff() { return stage_c0() * 32; }
+// acc += one stage (byte address wl of the stage plus stage_woff()) times the
+// input columns at xl (stage_xoff() included); chunks from ccn on hold another
+// stage's bytes.  Full stages take the branch-free path.
+__device__ __forceinline__ void stage_dot(RowAcc& acc, uint32_t wl, uint32_t xl, int ccn) {
+    auto chunk = [&](const uint4 (&wv)[4], int u) {
+        const float4 x0 = lds128f(xl + u * kStageStep * 32), x1 = lds128f(xl + u * kStageStep * 32 + 16);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            float2 t = acc.a[q];
+            t = fma2(make_float2(bflo(wv[q].x), bfhi(wv[q].x)), make_float2(x0.x, x0.y), t);
+            t = fma2(make_float2(bflo(wv[q].y), bfhi(wv[q].y)), make_float2(x0.z, x0.w), t);
+            t = fma2(make_float2(bflo(wv[q].z), bfhi(wv[q].z)), make_float2(x1.x, x1.y), t);
+            t = fma2(make_float2(bflo(wv[q].w), bfhi(wv[q].w)), make_float2(x1.z, x1.w), t);
+            acc.a[q] = t;
+        }
+    };
+    if (ccn == kColsPerChunk / 8) {
+        uint4 wv[kStageU][4];
+#pragma unroll
+        for (int u = 0; u < kStageU; ++u)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) wv[u][q] = lds128(wl + u * kStageStep * 512 + q * 128);
+#pragma unroll
+        for (int u = 0; u < kStageU; ++u) chunk(wv[u], u);
+        return;
+    }
+#pragma unroll 1
+    for (int u = 0; u < kStageU; ++u)
+        if (stage_c0() + u * kStageStep < ccn) {
+            uint4 wv[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) wv[q] = lds128(wl + u * kStageStep * 512 + q * 128);
+            chunk(wv, u);
+        }
 }
-
 
 // ------------------------------------------------------------ work geometry
 // Q/K/V and gate/up are split by whole 32-row tiles: rank r < Ge =
@@ -362,13 +394,16 @@ struct Smem {
     float* xa;          // [max items][512] staged input columns of the O / down items, then
                         // [max items][32] residual rows of the O items of chunk 0
     float2* rope;       // [D/2] (cos, sin) of the step's position
-    float* red;         // [2][kCW][32], then [kCW] sums of squares of the RMSNorm
+    float* red;         // [kRedSlots][kCW][32], then [kCW] sums of squares of the RMSNorm
     float* qa;          // [group][D] scaled queries of the attention unit
     float* kv;          // [2][D] k, v of the step's position
-    float* sc;          // [group][pps * page_size] scores, then probabilities
+    float* sc;          // [pps * page_size][sc_heads(group)] scores, then probabilities
     float* ml;          // [group][2] max, sum
     uint8_t* nsd;       // [down tiles] slots per down tile
 };
+// Heads of a score row: the group rounded up to 4, so that a position's
+// probabilities of four heads are one 16-byte load.
+__host__ __device__ constexpr int sc_heads(int grp) { return (grp + 3) & ~3; }
 __device__ __forceinline__ Smem carve(uint8_t* base, const DevModel& m, const SegPlan& p) {
     Smem s;
     uint8_t* q = base;
@@ -386,14 +421,14 @@ __device__ __forceinline__ Smem carve(uint8_t* base, const DevModel& m, const Se
     s.rope = reinterpret_cast<float2*>(f);
     f += m.D;
     s.red = f;
-    f += 2 * kCW * 32 + kCW;
+    f += kRedSlots * kCW * 32 + kCW;
     const int grp = m.A / m.KH;
     s.qa = f;
     f += grp * m.D;
     s.kv = f;
     f += 2 * m.D;
     s.sc = f;
-    f += grp * p.max_pps * m.page_size;
+    f += sc_heads(grp) * p.max_pps * m.page_size;
     s.ml = f;
     f += 2 * grp;
     s.nsd = reinterpret_cast<uint8_t*>(f);
@@ -677,31 +712,41 @@ __device__ __forceinline__ float gather_norm(float* xs, const uint16_t* g, int d
 }
 
 // Whole tiles [t0, t1) of a matrix with rows of length K against x (all K
-// columns in shared memory).  epi(t, s) runs in warp 0 with lane = row of
-// the tile and s its complete dot product.
+// columns in shared memory).  epi(t, s) runs in one warp with lane = row of
+// the tile and s its complete dot product.  The warps' partial sums of up to
+// kRedSlots tiles meet at one barrier and the epilogues run in different
+// warps: with a barrier and an epilogue in warp 0 for every tile, warp 0 held
+// up the other seven.  (Callers have a consumer barrier between one call's
+// epilogues and the next call.)
 template <class Epi>
-__device__ __forceinline__ void tile_gemv(Consumer& cs, int t0, int t1, int K, int nc, const float* x, float* red,
-                                          int& rb, Epi epi) {
+__device__ __forceinline__ void tile_gemv(Consumer& cs, int t0, int t1, int K, int nc, const float* x, float* red, Epi epi) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int t = t0; t < t1; ++t) {
-        float acc = 0.f;
-        for (int c = 0; c < nc; ++c) {
-            const uint32_t buf = saddr(cs.acquire()) + lane * 16 + w * 512;
-            const int ccn = (int)(chunk_bytes(K, c) / 512);
-            const uint32_t xc = saddr(x + c * kColsPerChunk) + w * 32;
-            if (cs.ok) acc += stage_dot<kCCPerWarp>(buf, xc, w, ccn);
-            cs.release();
+#pragma unroll 1
+    for (int tb = t0; tb < t1; tb += kRedSlots) {
+        const int te = min(t1, tb + kRedSlots);
+#pragma unroll 1
+        for (int t = tb; t < te; ++t) {
+            RowAcc acc;
+            acc.clear();
+#pragma unroll 1
+            for (int c = 0; c < nc; ++c) {
+                const uint32_t buf = saddr(cs.acquire()) + stage_woff();
+                const int ccn = (int)(chunk_bytes(K, c) / 512);
+                const uint32_t xc = saddr(x + c * kColsPerChunk) + stage_xoff();
+                if (cs.ok) stage_dot(acc, buf, xc, ccn);
+                cs.release();
+            }
+            red[(t - tb) * kCW * 32 + w * 32 + lane] = acc.total();
         }
-        float* r = red + rb * kCW * 32;
-        r[w * 32 + lane] = acc;
         csync();
-        if (w == 0) {
+        if (tb + w < te) {
+            const float* r = red + w * kCW * 32 + lane;
             float sum = 0.f;
 #pragma unroll
-            for (int k = 0; k < kCW; ++k) sum += r[k * 32 + lane];
-            epi(t, sum);
+            for (int k = 0; k < kCW; ++k) sum += r[k * 32];
+            epi(tb + w, sum);
         }
-        rb ^= 1;
+        if (te < t1) csync();
     }
 }
 
@@ -756,6 +801,235 @@ __device__ __forceinline__ float4 resid_mid4(const SegPlan& p, const Tagged* opa
     return v;
 }
 
+// The attention unit of one CTA: kv head g, cached positions [p0, p1) of
+// [0, pos], for the group's query heads; writes the split's unnormalised
+// output, maximum and sum per head.
+template <int D>
+__device__ __forceinline__ void attn_phase(const DevModel& m, const SegPlan& p, const Smem& s, Consumer& cs, Poll& pl,
+                                           const AttnGeo& ag, int unit, int pos, uint32_t tag) {
+    constexpr int kPairs = D / 32;  // pairs of k16 steps (32 dimensions)
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int grp = m.A / m.KH, gp = sc_heads(grp);
+    const int rpc = p.rows_per_kv_chunk;
+    const int g = unit / ag.splits, sp = unit - g * ag.splits;
+    const int p0 = sp * ag.pps * m.page_size, p1 = min(ag.T, min(ag.n_pages, (sp + 1) * ag.pps) * m.page_size);
+    const int npos = p1 - p0;
+    // ring stages of the unit's keys, and of its values (whole pages)
+    const int nst = (min(ag.n_pages, (sp + 1) * ag.pps) - sp * ag.pps) * (m.page_size / rpc);
+    pl.probe(p.kvn + (m.KH + g + 1) * D - 1, tag);  // the last value of this group's v
+    const Tagged* qsrc = p.q + (int64_t)g * grp * D;
+    const Tagged* kt = p.kvn + (int64_t)g * D;
+    const Tagged* vt = p.kvn + (int64_t)(m.KH + g) * D;
+    const int nqa = grp * D;
+    const float scale = 1.0f / sqrtf((float)D);
+    // The group's scaled queries as three bf16 parts (high + middle + low = q
+    // exactly) in rows padded to 16 bytes past D (xs is free here: seg_plan
+    // checks it holds 3 grp (D + 8) bf16), so that the fragment loads of 8
+    // heads at one column fall in different banks; then the step's k and v,
+    // all in one round of loads.
+    uint16_t* qhs = reinterpret_cast<uint16_t*>(s.xs);
+    constexpr int qrow = D + 8;
+#pragma unroll 1
+    for (int b = 4 * threadIdx.x; b < nqa + 2 * D; b += 4 * kCT) {
+        const Tagged* at = b < nqa ? qsrc + b : b < nqa + D ? kt + (b - nqa) : vt + (b - nqa - D);
+        uint32_t bad = 0;
+        float4 v = load4(at, tag, bad);
+        if (bad) {
+            Bound bd;
+            while (pl.again(bd)) {
+                bad = 0;
+                v = load4(at, tag, bad);
+                if (!bad) break;
+            }
+        }
+        if (b >= nqa) {
+            *reinterpret_cast<float4*>(s.kv + (b - nqa)) = v;
+        } else {
+            const int h = b / D, c = b - h * D;
+            uint32_t h01, m01, l01, h23, m23, l23;
+            split3_bf16x2(v.x * scale, v.y * scale, h01, m01, l01);
+            split3_bf16x2(v.z * scale, v.w * scale, h23, m23, l23);
+            sts64(saddr(qhs + h * qrow + c), h01, h23);
+            sts64(saddr(qhs + (grp + h) * qrow + c), m01, m23);
+            sts64(saddr(qhs + (2 * grp + h) * qrow + c), l01, l23);
+        }
+    }
+    csync();
+    // Scores on the tensor cores: S[h][r] = q_h . k_r as mma m16n8k16
+    // (bf16 operands, fp32 accumulation) with B = 8 cached keys and A the
+    // group's queries in three parts: one product with the high parts in rows
+    // 0..7 and the middle parts in rows 8..15, a second with the low parts in
+    // rows 0..7 (rows 8..15 zero), into the same accumulators.  The bf16
+    // products are exact in fp32.  A lane loads 8 consecutive dimensions of
+    // one key row (16 bytes, no bank conflicts beyond the row stride's); the
+    // product's k index runs over the dimensions in the same permuted order in
+    // A and B.  Row g of the result holds head g's high- and low-part dot
+    // products, row g + 8 its middle-part one.
+    const int g8 = lane >> 2, t4 = lane & 3;
+    {
+        // [pair][word]: dimensions pair*32 + 8 t4 .. +7 of query g8 (the low
+        // parts stay in shared memory: qlo_at, read with each product)
+        uint4 qhi[kPairs], qmid[kPairs];
+        const bool qrow_ok = g8 < grp;
+        const uint32_t q_at = saddr(qhs + (qrow_ok ? g8 : 0) * qrow + 8 * t4);
+        const uint32_t qlo_at = q_at + 2 * grp * qrow * 2;
+#pragma unroll
+        for (int pr = 0; pr < kPairs; ++pr) {
+            qhi[pr] = qrow_ok ? lds128(q_at + pr * 64) : make_uint4(0u, 0u, 0u, 0u);
+            qmid[pr] = qrow_ok ? lds128(q_at + grp * qrow * 2 + pr * 64) : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll 1
+        for (int st = 0; st < nst; ++st) {
+            const uint32_t kst = saddr(cs.acquire());
+            const int base = p0 + st * rpc, nr = min(rpc, p1 - base);
+            if (cs.ok) {
+#pragma unroll 1
+                for (int r0 = w * 8; r0 < nr; r0 += kCW * 8) {
+                    const int own = pos - base;
+                    if (own >= r0 && own < r0 + 8) {
+                        // the ring holds the cache's stale copy of the step's
+                        // own row: write the new k over it (bf16, exact)
+                        if (lane < D / 4) {
+                            const float4 kk = lds128f(saddr(s.kv + 4 * lane));
+                            sts64(kst + own * D * 2 + 8 * lane, pack_bf16x2(kk.x, kk.y), pack_bf16x2(kk.z, kk.w));
+                        }
+                        __syncwarp();
+                    }
+                    const uint32_t krow = kst + (r0 + g8) * D * 2 + 16 * t4;
+                    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                    for (int pr = 0; pr < kPairs; ++pr) {
+                        const uint4 kw = lds128(krow + pr * 64);
+                        mma_bf16(acc, qhi[pr].x, qmid[pr].x, qhi[pr].y, qmid[pr].y, kw.x, kw.y);
+                        mma_bf16(acc, qhi[pr].z, qmid[pr].z, qhi[pr].w, qmid[pr].w, kw.z, kw.w);
+                        uint4 lo = lds128(qlo_at + pr * 64);
+                        if (!qrow_ok) lo = make_uint4(0u, 0u, 0u, 0u);
+                        mma_bf16(acc, lo.x, 0u, lo.y, 0u, kw.x, kw.y);
+                        mma_bf16(acc, lo.z, 0u, lo.w, 0u, kw.z, kw.w);
+                    }
+                    const int ra = r0 + 2 * t4;
+                    if (qrow_ok) {
+                        float* sr = s.sc + (base - p0 + ra) * gp + g8;
+                        if (ra < nr) sr[0] = acc[0] + acc[2];
+                        if (ra + 1 < nr) sr[gp] = acc[1] + acc[3];
+                    }
+                }
+            }
+            // generic writes to the stage (the fixed row) before the
+            // producer's next bulk copy into it
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            cs.release();
+        }
+    }
+    csync();
+    // softmax statistics: warp = head
+    if (w < grp) {
+        float* sw = s.sc + w;
+        float mx = -INFINITY;
+#pragma unroll 1
+        for (int k = lane; k < npos; k += 32) mx = fmaxf(mx, sw[k * gp]);
+        mx = warp_max(mx);
+        float sum = 0.f;
+#pragma unroll 1
+        for (int k = lane; k < npos; k += 32) {
+            const float e = expf(sw[k * gp] - mx);
+            sw[k * gp] = e;
+            sum += e;
+        }
+        sum = warp_sum(sum);
+        if (lane == 0) {
+            s.ml[2 * w] = mx;
+            s.ml[2 * w + 1] = sum;
+        }
+    }
+    csync();
+    // P V: warp w takes the four heads from 4 hg on, hg = w / npq, and the
+    // positions r = w mod npq (mod npq); lane = dpl dimensions.  Each V row is
+    // read once per four heads, with one load for its four probabilities (those
+    // past the group are garbage, multiplied into sums nobody reads).  The npq
+    // partial sums per head meet in shared memory (xs and xa, contiguous and
+    // free here) and are added in order.
+    constexpr int dpl = D / 32;  // 2 or 4
+    const int avail = ((max(m.d, m.A * D) + 3) & ~3) + p.max_items * (kColsPerChunk + 32);
+    int npq = kCW / (gp >> 2);
+#pragma unroll 1
+    while (npq > 1 && npq * grp * D > avail) npq >>= 1;
+    const int hg = w / npq, pq = w - hg * npq;
+    const bool pv = hg * 4 < grp;
+    float acc[4][dpl];
+#pragma unroll
+    for (int hh = 0; hh < 4; ++hh)
+#pragma unroll
+        for (int k = 0; k < dpl; ++k) acc[hh][k] = 0.f;
+#pragma unroll 1
+    for (int st = 0; st < nst; ++st) {
+        const uint32_t vst = saddr(cs.acquire());
+        const int base = p0 + st * rpc, nr = min(rpc, p1 - base), own = pos - base;
+        if (pv && cs.ok) {
+            if (own >= 0 && own < nr && own % npq == pq) {
+                // the step's own v over its stale row (the warps that read it
+                // write the same bytes)
+                if (lane < D / 4) {
+                    const float4 vv = lds128f(saddr(s.kv + D + 4 * lane));
+                    sts64(vst + own * D * 2 + 8 * lane, pack_bf16x2(vv.x, vv.y), pack_bf16x2(vv.z, vv.w));
+                }
+                __syncwarp();
+            }
+            const uint32_t va = vst + lane * dpl * 2, pa = saddr(s.sc + (base - p0) * gp + hg * 4);
+#pragma unroll 4
+            for (int r = pq; r < nr; r += npq) {
+                const float4 pr = lds128f(pa + r * gp * 4);
+                float v[dpl];
+                if (dpl == 4) {
+                    const uint2 u = lds64(va + r * D * 2);
+                    v[0] = bflo(u.x), v[1] = bfhi(u.x), v[dpl - 2] = bflo(u.y), v[dpl - 1] = bfhi(u.y);
+                } else {
+                    const uint32_t u = lds32(va + r * D * 2);
+                    v[0] = bflo(u), v[1] = bfhi(u);
+                }
+                const float pp[4] = {pr.x, pr.y, pr.z, pr.w};
+#pragma unroll
+                for (int hh = 0; hh < 4; ++hh)
+#pragma unroll
+                    for (int k = 0; k < dpl; ++k) acc[hh][k] = fmaf(pp[hh], v[k], acc[hh][k]);
+            }
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        cs.release();
+    }
+    float* part = s.xs;  // [grp][npq][D]
+    if (pv) {
+#pragma unroll
+        for (int hh = 0; hh < 4; ++hh) {
+            const int h = hg * 4 + hh;
+            if (h < grp) {
+                float* dst = part + (h * npq + pq) * D + lane * dpl;
+#pragma unroll
+                for (int k = 0; k < dpl; ++k) dst[k] = acc[hh][k];
+            }
+        }
+    }
+    csync();
+#pragma unroll 1
+    for (int e = threadIdx.x; e < grp * (D / 4); e += kCT) {
+        const int h = e / (D / 4), c = 4 * (e % (D / 4));
+        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+        for (int k = 0; k < npq; ++k) sum = f4add(sum, *reinterpret_cast<const float4*>(part + (h * npq + k) * D + c));
+        Tagged* dst = p.attn_part + ((int64_t)(g * grp + h) * kSegMaxSplits + sp) * (D + 4) + c;
+        st_tagged(dst, sum.x, tag);
+        st_tagged(dst + 1, sum.y, tag);
+        st_tagged(dst + 2, sum.z, tag);
+        st_tagged(dst + 3, sum.w, tag);
+    }
+    if (threadIdx.x < grp) {
+        Tagged* dst = p.attn_part + ((int64_t)(g * grp + threadIdx.x) * kSegMaxSplits + sp) * (D + 4) + D;
+        st_tagged(dst, s.ml[2 * threadIdx.x], tag);
+        st_tagged(dst + 1, s.ml[2 * threadIdx.x + 1], tag);
+    }
+    csync();  // xs and xa are read: the O phase may write them
+}
+
 }  // namespace
 
 __global__ void __launch_bounds__(kSegThreads, 1) k_layers(DevModel m, SegPlan p, int j0, int j1, int first) {
@@ -763,8 +1037,7 @@ __global__ void __launch_bounds__(kSegThreads, 1) k_layers(DevModel m, SegPlan p
     const Smem s = carve(seg_smem, m, p);
     const int cta = blockIdx.x, G = p.G;
     const Waits wt{&m.ctl->err, p.stall_cycles, p.check_cycles};
-    const int half = m.D >> 1, grp = m.A / m.KH;
-    const int AD = m.A * m.D;
+    const int half = m.D >> 1;
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < p.stages; ++i) {
@@ -867,7 +1140,6 @@ __global__ void __launch_bounds__(kSegThreads, 1) k_layers(DevModel m, SegPlan p
     const unsigned seq0 = sync[1];  // layers run since the context was reset
     for (int i = threadIdx.x; i < half; i += kCT) s.rope[i] = m.rope[(int64_t)pos * half + i];
     const float2* cs_row = s.rope;
-    const float scale = 1.0f / sqrtf((float)m.D);
     const int slice0 = (int)((int64_t)cta * m.d / G), slice1 = (int)((int64_t)(cta + 1) * m.d / G);
     const int nq = m.A * half, nk = m.KH * half;
     const int64_t kvo_pos = ((int64_t)m.page_table[pos / m.page_size] * m.KH * m.page_size + pos % m.page_size) * m.D;
@@ -926,12 +1198,12 @@ __global__ void __launch_bounds__(kSegThreads, 1) k_layers(DevModel m, SegPlan p
                 pl.probe(p.dpart + (last_dn_slot + s.nsd[p.n_tiles[3] - 1] - 1) * 32 + 31, seq_tag(seq - 1));
             else
                 csync();
-            const float inv = gather_norm<2>(s.xs, lw + m.off_gattn, m.d, m.eps, s.red + 2 * kCW * 32, pl,
+            const float inv = gather_norm<2>(s.xs, lw + m.off_gattn, m.d, m.eps, s.red + kRedSlots * kCW * 32, pl,
                                           [&](int i, uint32_t& bad) { return rin.four(i, bad); });
             const uint16_t* bias = m.qkv_bias ? lw + m.off_bqkv : nullptr;
             uint16_t* kdst = m.kpool + (int64_t)j * m.kv_layer_stride + kvo_pos;
             uint16_t* vdst = m.vpool + (int64_t)j * m.kv_layer_stride + kvo_pos;
-            tile_gemv(cs, tq0, tq1, p.K[0], p.n_chunks[0], s.xs, s.red, rb, [&](int t, float v) {
+            tile_gemv(cs, tq0, tq1, p.K[0], p.n_chunks[0], s.xs, s.red, [&](int t, float v) {
                 const int odd = lane & 1;
                 const int u = t * 16 + (lane >> 1);
                 v *= inv;
@@ -969,228 +1241,10 @@ __global__ void __launch_bounds__(kSegThreads, 1) k_layers(DevModel m, SegPlan p
 
         // ---------------- attention unit (if this CTA has one)
         if (unit >= 0) {
-            const int g = unit / ag.splits, sp = unit - g * ag.splits;
-            const int pg0 = sp * ag.pps, pg1 = min(ag.n_pages, pg0 + ag.pps);
-            const int p0 = pg0 * m.page_size, p1 = min(ag.T, pg1 * m.page_size);
-            const int npos = p1 - p0;
-            pl.probe(p.kvn + (m.KH + g + 1) * m.D - 1, tag);  // the last value of this group's v
-            const Tagged* qsrc = p.q + (int64_t)g * grp * m.D;
-            const Tagged* kt = p.kvn + (int64_t)g * m.D;
-            const Tagged* vt = p.kvn + (int64_t)(m.KH + g) * m.D;
-            // the group's scaled queries, then k and v, in one round (s.kv follows s.qa)
-            const int nqa = grp * m.D;
-            gather4<1>(s.qa, nqa + 2 * m.D, pl, [&](int i, uint32_t& bad) {
-                if (i >= nqa) {
-                    const int e = i - nqa;
-                    return load4(e < m.D ? kt + e : vt + e - m.D, tag, bad);
-                }
-                const float4 q = load4(qsrc + i, tag, bad);
-                return make_float4(q.x * scale, q.y * scale, q.z * scale, q.w * scale);
-            });
-            csync();
-            // Scores on the tensor cores: S[h][r] = q_h . k_r as mma m16n8k16
-            // (bf16 operands, fp32 accumulation) with B = 8 cached keys and A
-            // the group's queries split into three bf16 parts (high + middle +
-            // low = q exactly): one product with the high parts in rows 0..7
-            // and the middle parts in rows 8..15, a second with the low parts
-            // in rows 0..7 (rows 8..15 zero), into the same accumulators.  The
-            // bf16 products are exact in fp32.  A lane loads 8 consecutive
-            // dimensions of one key row (16 bytes, no bank conflicts beyond the
-            // row stride's); the product's k index runs over the dimensions in
-            // the same permuted order in A and B.  Row g of the result holds
-            // head g's high- and low-part dot products, row g + 8 its
-            // middle-part one.
-            const int spc = p.max_pps * m.page_size;  // score row stride
-            const int npair = m.D >> 5;               // pairs of k16 steps (32 dimensions)
-            const int g8 = lane >> 2, t4 = lane & 3;
-            // The group's queries as three bf16 parts, converted once into
-            // rows padded to 16 bytes past D (xs is free here: seg_plan checks
-            // it holds 3 grp (D + 8) bf16), so that the fragment loads of 8
-            // heads at one column fall in different banks.
-            {
-                const int qrow = m.D + 8;
-                uint16_t* qhs = reinterpret_cast<uint16_t*>(s.xs);
-                for (int e = threadIdx.x; e < nqa / 4; e += kCT) {
-                    const float4 q4 = lds128f(saddr(s.qa + 4 * e));
-                    const int h = (4 * e) / m.D, c = 4 * e - h * m.D;
-                    uint32_t h01, m01, l01, h23, m23, l23;
-                    split3_bf16x2(q4.x, q4.y, h01, m01, l01);
-                    split3_bf16x2(q4.z, q4.w, h23, m23, l23);
-                    sts64(saddr(qhs + h * qrow + c), h01, h23);
-                    sts64(saddr(qhs + (grp + h) * qrow + c), m01, m23);
-                    sts64(saddr(qhs + (2 * grp + h) * qrow + c), l01, l23);
-                }
-                csync();
-            }
-            // [pair][word]: dimensions pair*32 + 8 t4 .. +7 of query g8 (the
-            // low parts stay in shared memory: qlo_at, read with each product)
-            uint32_t qhi[4][4], qmid[4][4];
-            const bool qrow_ok = g8 < grp;
-            const uint32_t qlo_at =
-                saddr(reinterpret_cast<const uint16_t*>(s.xs) + (2 * grp + (qrow_ok ? g8 : 0)) * (m.D + 8) + 8 * t4);
-#pragma unroll
-            for (int pr = 0; pr < 4; ++pr) {
-                if (pr < npair && qrow_ok) {
-                    const uint16_t* qhs = reinterpret_cast<const uint16_t*>(s.xs) + g8 * (m.D + 8) + pr * 32 + 8 * t4;
-                    const uint4 a = lds128(saddr(qhs)), b = lds128(saddr(qhs + grp * (m.D + 8)));
-                    qhi[pr][0] = a.x, qhi[pr][1] = a.y, qhi[pr][2] = a.z, qhi[pr][3] = a.w;
-                    qmid[pr][0] = b.x, qmid[pr][1] = b.y, qmid[pr][2] = b.z, qmid[pr][3] = b.w;
-                } else {
-#pragma unroll
-                    for (int wd = 0; wd < 4; ++wd) qhi[pr][wd] = qmid[pr][wd] = 0u;
-                }
-            }
-            for (int pg = pg0; pg < pg1; ++pg)
-                for (int q = 0; q < cpp; ++q) {
-                    const uint32_t kst = saddr(cs.acquire());
-                    const int base = pg * m.page_size + q * rpc;
-                    const int nr = min(rpc, p1 - base);
-                    if (cs.ok) {
-                        for (int nt = w; nt * 8 < nr; nt += kCW) {
-                            const int r0 = nt * 8, own = pos - base;
-                            if (own >= r0 && own < r0 + 8) {
-                                // the ring holds the cache's stale copy of the step's
-                                // own row: write the new k over it (bf16, exact)
-                                for (int e = lane; e < (m.D >> 2); e += 32) {
-                                    const float4 kk = lds128f(saddr(s.kv + 4 * e));
-                                    sts64(kst + own * m.D * 2 + 8 * e, pack_bf16x2(kk.x, kk.y), pack_bf16x2(kk.z, kk.w));
-                                }
-                                __syncwarp();
-                            }
-                            const uint32_t krow = kst + (r0 + g8) * m.D * 2 + 16 * t4;
-                            float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                            for (int pr = 0; pr < 4; ++pr) {
-                                if (pr < npair) {
-                                    const uint4 kw = lds128(krow + pr * 64);
-                                    mma_bf16(acc, qhi[pr][0], qmid[pr][0], qhi[pr][1], qmid[pr][1], kw.x, kw.y);
-                                    mma_bf16(acc, qhi[pr][2], qmid[pr][2], qhi[pr][3], qmid[pr][3], kw.z, kw.w);
-                                    uint4 lo = lds128(qlo_at + pr * 64);
-                                    if (!qrow_ok) lo = make_uint4(0u, 0u, 0u, 0u);
-                                    mma_bf16(acc, lo.x, 0u, lo.y, 0u, kw.x, kw.y);
-                                    mma_bf16(acc, lo.z, 0u, lo.w, 0u, kw.z, kw.w);
-                                }
-                            }
-                            const int ra = r0 + 2 * t4;
-                            if (g8 < grp) {
-                                float* sr = s.sc + g8 * spc + (base - p0);
-                                if (ra < nr) sr[ra] = acc[0] + acc[2];
-                                if (ra + 1 < nr) sr[ra + 1] = acc[1] + acc[3];
-                            }
-                        }
-                    }
-                    // generic writes to the stage (the fixed row) before the
-                    // producer's next bulk copy into it
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    cs.release();
-                }
-            csync();
-            for (int hh = w; hh < grp; hh += kCW) {
-                float mx = -INFINITY;
-                for (int k = lane; k < npos; k += 32) mx = fmaxf(mx, s.sc[hh * spc + k]);
-                mx = warp_max(mx);
-                float sum = 0.f;
-                for (int k = lane; k < npos; k += 32) {
-                    const float e = expf(s.sc[hh * spc + k] - mx);
-                    s.sc[hh * spc + k] = e;
-                    sum += e;
-                }
-                sum = warp_sum(sum);
-                if (lane == 0) {
-                    s.ml[2 * hh] = mx;
-                    s.ml[2 * hh + 1] = sum;
-                }
-            }
-            csync();
-            // P V: warp w takes head group hg = w / npq (hpg heads) and the
-            // positions r = w mod npq (mod npq); lane = dpl dimensions.  Each V
-            // row is read once per head group.  The npq partial sums per head
-            // meet in shared memory (xs and xa, contiguous and free here) and are
-            // added in order.
-            const int dpl = m.D >> 5;  // 2 or 4
-            const int hgn = grp > 4 ? 2 : 1, hpg = (grp + hgn - 1) / hgn;
-            const int avail = ((max(m.d, AD) + 3) & ~3) + p.max_items * (kColsPerChunk + 32);
-            int npq = kCW / hgn;
-            while (npq > 1 && npq * grp * m.D > avail) npq >>= 1;
-            const int hg = w / npq, pq = w - hg * npq;
-            const bool pv = hg < hgn;
-            float vvt[4];  // the step's own v (this lane's dimensions)
-            if (dpl == 4) {
-                const float4 t = lds128f(saddr(s.kv + m.D + lane * 4));
-                vvt[0] = t.x, vvt[1] = t.y, vvt[2] = t.z, vvt[3] = t.w;
-            } else {
-                const float2 t = *reinterpret_cast<const float2*>(s.kv + m.D + lane * 2);
-                vvt[0] = t.x, vvt[1] = t.y, vvt[2] = vvt[3] = 0.f;
-            }
-            float acc[4][4];
-#pragma unroll
-            for (int hh = 0; hh < 4; ++hh)
-#pragma unroll
-                for (int k = 0; k < 4; ++k) acc[hh][k] = 0.f;
-            for (int pg = pg0; pg < pg1; ++pg)
-                for (int q = 0; q < cpp; ++q) {
-                    const uint32_t vb = saddr(cs.acquire()) + lane * dpl * 2;
-                    const int base = pg * m.page_size + q * rpc;
-                    const int nr = min(rpc, p1 - base);
-                    if (pv && cs.ok) {
-                        const float* pr0 = s.sc + (hg * hpg) * spc + (base - p0);
-#pragma unroll 4
-                        for (int r = pq; r < nr; r += npq) {
-                            float v[4];
-                            if (dpl == 4) {
-                                const uint2 u = lds64(vb + r * m.D * 2);
-                                v[0] = bflo(u.x), v[1] = bfhi(u.x), v[2] = bflo(u.y), v[3] = bfhi(u.y);
-                            } else {
-                                const uint32_t u = lds32(vb + r * m.D * 2);
-                                v[0] = bflo(u), v[1] = bfhi(u), v[2] = v[3] = 0.f;
-                            }
-                            const bool own = base + r == pos;  // the ring's copy of this row is stale
-#pragma unroll
-                            for (int k = 0; k < 4; ++k) v[k] = own ? vvt[k] : v[k];
-#pragma unroll
-                            for (int hh = 0; hh < 4; ++hh) {
-                                if (hh < hpg && hg * hpg + hh < grp) {
-                                    const float pr = pr0[hh * spc + r];
-#pragma unroll
-                                    for (int k = 0; k < 4; ++k) acc[hh][k] = fmaf(pr, v[k], acc[hh][k]);
-                                }
-                            }
-                        }
-                    }
-                    cs.release();
-                }
-            float* part = s.xs;  // [grp][npq][D]
-            if (pv) {
-#pragma unroll
-                for (int hh = 0; hh < 4; ++hh) {
-                    const int h = hg * hpg + hh;
-                    if (hh < hpg && h < grp) {
-                        float* dst = part + (h * npq + pq) * m.D + lane * dpl;
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            if (k < dpl) dst[k] = acc[hh][k];
-                    }
-                }
-            }
-            csync();
-            {
-                const int d4 = m.D >> 2;
-                for (int e = threadIdx.x; e < grp * d4; e += kCT) {
-                    const int h = e / d4, c = 4 * (e - h * d4);
-                    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-                    for (int k = 0; k < npq; ++k) sum = f4add(sum, *reinterpret_cast<const float4*>(part + (h * npq + k) * m.D + c));
-                    Tagged* dst = p.attn_part + ((int64_t)(g * grp + h) * kSegMaxSplits + sp) * (m.D + 4) + c;
-                    st_tagged(dst, sum.x, tag);
-                    st_tagged(dst + 1, sum.y, tag);
-                    st_tagged(dst + 2, sum.z, tag);
-                    st_tagged(dst + 3, sum.w, tag);
-                }
-                if (threadIdx.x < grp) {
-                    Tagged* dst = p.attn_part + ((int64_t)(g * grp + threadIdx.x) * kSegMaxSplits + sp) * (m.D + 4) + m.D;
-                    st_tagged(dst, s.ml[2 * threadIdx.x], tag);
-                    st_tagged(dst + 1, s.ml[2 * threadIdx.x + 1], tag);
-                }
-            }
+            if (m.D == 128)
+                attn_phase<128>(m, p, s, cs, pl, ag, unit, pos, tag);
+            else
+                attn_phase<64>(m, p, s, cs, pl, ag, unit, pos, tag);
         }
 
         // ---------------- O items: merge the attention splits of the chunk's heads,
@@ -1316,15 +1370,18 @@ __global__ void __launch_bounds__(kSegThreads, 1) k_layers(DevModel m, SegPlan p
                 *dst = make_float2(num.x * inv, num.y * inv);
             }
             csync();
+#pragma unroll 1
             for (int i = io.lo; i < io.hi; ++i) {
                 const int t = i / io.nc, ch = i - t * io.nc;
-                const uint32_t buf = saddr(cs.acquire()) + lane * 16 + w * 512;
+                const uint32_t buf = saddr(cs.acquire()) + stage_woff();
                 const int ccn = (int)(chunk_bytes(io.K, ch) / 512);
-                const uint32_t x = saddr(s.xa + (i - io.lo) * kColsPerChunk) + w * 32;
-                const float acc = cs.ok ? stage_dot<kCCPerWarp>(buf, x, w, ccn) : 0.f;
+                const uint32_t x = saddr(s.xa + (i - io.lo) * kColsPerChunk) + stage_xoff();
+                RowAcc acc;
+                acc.clear();
+                if (cs.ok) stage_dot(acc, buf, x, ccn);
                 cs.release();
                 float* r = s.red + rb * kCW * 32;
-                r[w * 32 + lane] = acc;
+                r[w * 32 + lane] = acc.total();
                 csync();
                 if (w == 0) {
                     float sum = ch == 0 ? rows[(i - io.lo) * 32 + lane] : 0.f;
@@ -1339,9 +1396,9 @@ __global__ void __launch_bounds__(kSegThreads, 1) k_layers(DevModel m, SegPlan p
         // ---------------- gate/up tiles: RMSNorm of the mid residual, SwiGLU
         if (tg1 > tg0) {
             pl.probe(op_cur + ((int64_t)p.n_tiles[1] * p.n_chunks[1] - 1) * 32 + 31, tag);  // the last O slot
-            const float inv = gather_norm<2>(s.xs, lw + m.off_gmlp, m.d, m.eps, s.red + 2 * kCW * 32, pl,
+            const float inv = gather_norm<2>(s.xs, lw + m.off_gmlp, m.d, m.eps, s.red + kRedSlots * kCW * 32, pl,
                                           [&](int i, uint32_t& bad) { return resid_mid4(p, op_cur, i, tag, bad); });
-            tile_gemv(cs, tg0, tg1, p.K[2], p.n_chunks[2], s.xs, s.red, rb, [&](int t, float v) {
+            tile_gemv(cs, tg0, tg1, p.K[2], p.n_chunks[2], s.xs, s.red, [&](int t, float v) {
                 v *= inv;
                 const float up = __shfl_xor_sync(0xffffffffu, v, 1);
                 const int f = t * 16 + (lane >> 1);
@@ -1379,18 +1436,20 @@ __global__ void __launch_bounds__(kSegThreads, 1) k_layers(DevModel m, SegPlan p
                 return f < m.F ? load4(p.a + f, tag, bad) : make_float4(0.f, 0.f, 0.f, 0.f);
             });
             csync();
-            float acc = 0.f;
+            RowAcc acc;
+            acc.clear();
+#pragma unroll 1
             for (int i = idn.lo; i < idn.hi; ++i) {
                 const int t = i / idn.nc, ch = i - t * idn.nc;
-                const uint32_t buf = saddr(cs.acquire()) + lane * 16 + w * 512;
+                const uint32_t buf = saddr(cs.acquire()) + stage_woff();
                 const int ccn = (int)(chunk_bytes(idn.K, ch) / 512);
-                const uint32_t x = saddr(s.xa + (i - idn.lo) * kColsPerChunk) + w * 32;
-                if (cs.ok) acc += stage_dot<kCCPerWarp>(buf, x, w, ccn);
+                const uint32_t x = saddr(s.xa + (i - idn.lo) * kColsPerChunk) + stage_xoff();
+                if (cs.ok) stage_dot(acc, buf, x, ccn);
                 cs.release();
                 if (i + 1 == idn.hi || ch + 1 == idn.nc) {
                     float* r = s.red + rb * kCW * 32;
-                    r[w * 32 + lane] = acc;
-                    acc = 0.f;
+                    r[w * 32 + lane] = acc.total();
+                    acc.clear();
                     csync();
                     if (w == 0) {
                         const int slot = cta - item_owner(idn, t * idn.nc);
@@ -1445,8 +1504,8 @@ __global__ void __launch_bounds__(kSegThreads, 1) k_vocab_ring(VocabArgs v, int 
     s.full = reinterpret_cast<uint64_t*>(vr_smem + (size_t)stages * kSegChunk);
     s.empty = s.full + stages;
     float* xs = reinterpret_cast<float*>(s.empty + stages);
-    float* red = xs + ((v.d + 3) & ~3);      // [2][kCW][32], then [kCW] norm partials
-    float* part = red + 2 * kCW * 32 + kCW;  // [d / 8] partial dot products of one row
+    float* red = xs + ((v.d + 3) & ~3);              // [kRedSlots][kCW][32], then [kCW] norm partials
+    float* part = red + kRedSlots * kCW * 32 + kCW;  // [d / 8] partial dot products of one row
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         err_local = 0;
@@ -1480,11 +1539,11 @@ __global__ void __launch_bounds__(kSegThreads, 1) k_vocab_ring(VocabArgs v, int 
     float ss = 0.f;
     for (int i = threadIdx.x; i < v.d; i += kCT) ss = fmaf(v.x[i], v.x[i], ss);
     ss = warp_sum(ss);
-    if (lane == 0) red[2 * kCW * 32 + w] = ss;
+    if (lane == 0) red[kRedSlots * kCW * 32 + w] = ss;
     csync();
     float tot = 0.f;
 #pragma unroll
-    for (int k = 0; k < kCW; ++k) tot += red[2 * kCW * 32 + k];
+    for (int k = 0; k < kCW; ++k) tot += red[kRedSlots * kCW * 32 + k];
     const float inv = 1.0f / sqrtf(tot / (float)v.d + v.eps);
     for (int i = threadIdx.x; i < v.d; i += kCT) xs[i] = v.x[i] * inv * bf(v.gain[i]);
     csync();
@@ -1511,32 +1570,14 @@ __global__ void __launch_bounds__(kSegThreads, 1) k_vocab_ring(VocabArgs v, int 
         lx = lx_s;
     }
     const bool keep = v.logits && (!v.logits_if_dbg || (v.ctl && v.ctl->dbg));
-    SoftStats st;
-    int rb = 0;
-    for (int t = t0; t < t1; ++t) {
-        float acc = 0.f;
-        for (int c = 0; c < nc; ++c) {
-            const uint32_t buf = saddr(cs.acquire()) + lane * 16 + w * 512;
-            const int ccn = (int)(chunk_bytes(v.d, c) / 512);
-            const uint32_t xc = saddr(xs + c * kColsPerChunk) + w * 32;
-            if (cs.ok) acc += stage_dot<kCCPerWarp>(buf, xc, w, ccn);
-            cs.release();
+    SoftStats st;  // warp w keeps the statistics of the tiles whose rows it finishes
+    tile_gemv(cs, t0, t1, v.d, nc, xs, red, [&](int t, float sum) {
+        const int row = t * kTileRows + lane;
+        if (row < v.V) {
+            if (keep) v.logits[row] = sum;
+            st.add(sum, row, lx, nx);
         }
-        float* r = red + rb * kCW * 32;
-        r[w * 32 + lane] = acc;
-        csync();
-        if (w == 0) {
-            float sum = 0.f;
-#pragma unroll
-            for (int k = 0; k < kCW; ++k) sum += r[k * 32 + lane];
-            const int row = t * kTileRows + lane;
-            if (row < v.V) {
-                if (keep) v.logits[row] = sum;
-                st.add(sum, row, lx, nx);
-            }
-        }
-        rb ^= 1;
-    }
+    });
     vocab_finish(v, st, nucleus, kCW, [] { csync(); });
 }
 
@@ -1665,7 +1706,7 @@ __global__ void __launch_bounds__(kSegThreads, 1) k_vocab_rows(VocabArgs v, int 
 
 bool vocab_ring_plan(int d, int n_sm, VocabRing& vr) {
     if (d % 8 || d <= 0 || n_sm <= 0) return false;
-    const size_t fixed = (size_t)(((d + 3) & ~3) + 2 * kCW * 32 + kCW + d / 8) * 4 + 1024;
+    const size_t fixed = (size_t)(((d + 3) & ~3) + kRedSlots * kCW * 32 + kCW + d / 8) * 4 + 1024;
     const size_t budget = 227 * 1024;
     if (fixed + 4 * (size_t)(kSegChunk + 16) > budget) return false;
     vr.G = n_sm;
@@ -1739,8 +1780,8 @@ bool seg_plan(const DevModel& m, int n_sm, SegPlan& p) {
     p.max_splits = std::min(cap, np_max);
     // xs, xa, rope, red (+ norm partials), qa, kv, sc, ml (the carve above)
     const size_t floats = (size_t)((std::max(m.d, m.A * m.D) + 3) & ~3) + (size_t)p.max_items * (kColsPerChunk + 32) +
-                          (size_t)m.D + 2 * kCW * 32 + kCW + (size_t)grp * m.D + 2 * (size_t)m.D +
-                          (size_t)grp * p.max_pps * m.page_size + 2 * (size_t)grp;
+                          (size_t)m.D + kRedSlots * kCW * 32 + kCW + (size_t)grp * m.D + 2 * (size_t)m.D +
+                          (size_t)sc_heads(grp) * p.max_pps * m.page_size + 2 * (size_t)grp;
     const size_t fixed = floats * 4 + (size_t)p.n_tiles[3] + 256;
     const size_t budget = 227 * 1024;
     if (fixed + 4 * (size_t)(kSegChunk + 16) > budget) return false;
