@@ -338,6 +338,7 @@ bool weight_map(CUtensorMap* map, const uint16_t* W, int64_t n_tiles, int K) {
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+bool small_batch(int M) { return x3_rows(M) <= USmall::EW / 4 * USmall::HC; }
 size_t umma_smem() { return (size_t)kUStages * kUStageBytes + 256 + 1024; }
 
 }  // namespace
@@ -363,12 +364,20 @@ bool umma_available() {
 }
 
 // K splits: as many as keep the grid within one wave (one CTA per SM: the
-// stages take most of the shared memory), at most one per stage.
+// stages take most of the shared memory), at most one per stage.  A small batch
+// (USmall) waits for latencies, not for the tensor cores: a split more shortens
+// every CTA's run of stages and lengthens the sum that the next launch starts
+// with, each by about the same time, so there are at most sqrt(2 stages) of
+// them.  A 33-position prompt at 0.5B (21 splits of two stages or fewer became
+// 7 of four, 21 of seven became 17 of nine): 1300 us before, 1254 now; 1262 with
+// sqrt(stages) splits, 1263 with sqrt(4 stages).
 int umma_splits(int64_t n_tiles, int K, int M, int n_sm) {
     const int64_t mt = (n_tiles + 3) / 4 * rows_blocks(M);
     const int nk = (K + kUKStage - 1) / kUKStage;
-    const int64_t want = n_sm / mt;
-    return (int)std::max<int64_t>(1, std::min<int64_t>(want, nk));
+    int64_t want = std::min<int64_t>(n_sm / mt, nk);
+    if (small_batch(M))
+        while (want * want > 2 * nk) --want;
+    return (int)std::max<int64_t>(1, want);
 }
 
 cudaError_t launch_mm_umma(const uint16_t* W, int64_t n_rows, int K, const uint16_t* x3, int ldx, int M, int S, float* part,
@@ -379,7 +388,7 @@ cudaError_t launch_mm_umma(const uint16_t* W, int64_t n_rows, int K, const uint1
     const dim3 grid((unsigned)((nt + 3) / 4), (unsigned)S, (unsigned)rows_blocks(M));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
-    const bool small = x3_rows(M) <= USmall::EW / 4 * USmall::HC;
+    const bool small = small_batch(M);
     cfg.blockDim = dim3(small ? USmall::threads : ULarge::threads);
     cfg.dynamicSmemBytes = umma_smem();
     cfg.stream = s;
