@@ -16,7 +16,7 @@
 //
 // CTA (x, s, z): weight rows [128 x, 128 x + 128) (four 32-row tiles) over the
 // K range of split s for row block z, 32 columns per pipeline stage, four
-// stages in flight:
+// stages in flight (eight for a small batch, whose stages are 20 KB):
 //   - the producer warp's lane 0 loads a stage: the 128 x 32 weight block with one TMA
 //     tensor copy (a three-dimensional view of the tile-packed layout whose
 //     box lands in shared memory in the UMMA canonical K-major layout with
@@ -58,33 +58,38 @@
 namespace ee {
 namespace {
 
+constexpr int kUMRows = 128;                        // weight rows per CTA (UMMA M)
+constexpr int kUKStage = 32;                        // K columns per stage
+constexpr int kUABytes = kUMRows * kUKStage * 2;    // 8 KB
+
 // A launch's shape.  EW epilogue warps read the accumulators (warp w:
 // tensor-memory lanes 32 (w mod 4), columns from HC (w / 4) on), then come the
 // producer warp and the MMA warp; CH stages of the high parts' products (at
 // most) add up in tensor memory.
-template <int EW_, int HC_, int CH_>
+template <int EW_, int HC_, int CH_, int ST_>
 struct UShape {
-    static constexpr int EW = EW_, HC = HC_, CH = CH_;
+    static constexpr int EW = EW_, HC = HC_, CH = CH_, ST = ST_;
     static constexpr int threads = 32 * (EW + 2);
+    static constexpr int rows = EW / 4 * HC;  // a block's rows, at most
+    // a stage: the weight block and the activations of a full block (8 + 48, 8 + 12 KB)
+    static constexpr int stage_bytes = kUABytes + kUKStage / 8 * 3 * rows * 16;
+    static constexpr int tmem_cols = 2 * rows;  // two accumulators of one fp32 column per position
+    static constexpr size_t smem = (size_t)ST * stage_bytes + 256 + 1024;
 };
-using ULarge = UShape<8, kRowsBlock / 2, 4>;
+using ULarge = UShape<8, kRowsBlock / 2, 4, 4>;
 // A small batch: fewer threads and registers, so that the launches before and
 // after find room beside it (programmatic launch), and longer chains, since its
-// products are too short to run under a read-back.
-using USmall = UShape<4, 64, 24>;
-constexpr int kUStages = 4;
-constexpr int kUMRows = 128;                        // weight rows per CTA (UMMA M)
-constexpr int kUKStage = 32;                        // K columns per stage
-constexpr int kUABytes = kUMRows * kUKStage * 2;    // 8 KB
-constexpr int kUBBytes = kUKStage / 8 * 3 * kRowsBlock * 16;  // a full block's activations: 48 KB
-constexpr int kUStageBytes = kUABytes + kUBBytes;   // 56 KB
-constexpr int kUTmemCols = 2 * kRowsBlock;          // two accumulators of one fp32 column per position
+// products are too short to run under a read-back.  Eight of its small stages,
+// so that most splits have their whole range in flight at once, the weights
+// since before the programmatic wait (33 positions at 0.5B: 1254 us with four
+// stages as long as a full block's, 1267 with four short ones, 1244 with eight).
+using USmall = UShape<4, 64, 24, 8>;
 
 // ---------------------------------------------------------------- copies
 __device__ __forceinline__ void u_expect_tx(uint64_t* bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(u_saddr(bar)), "r"(bytes) : "memory");
 }
-// The 128 x 64 weight block at (tile t0, 16-byte column chunk c0) of the
+// The 128 x 32 weight block at (tile t0, 16-byte column chunk c0) of the
 // three-dimensional view {256 elements (one chunk of a 32-row tile), tiles,
 // chunks}.
 __device__ __forceinline__ void u_tma_w(void* dst, const CUtensorMap* map, int t0, int c0, uint64_t* bar) {
@@ -107,9 +112,9 @@ __global__ void __launch_bounds__(U::threads, 1)
                 int M_all, int S, float* __restrict__ part, int Np, int* err) {
     extern __shared__ __align__(1024) uint8_t u_smem_raw[];
     uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(u_smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint64_t* full = reinterpret_cast<uint64_t*>(sm + kUStages * kUStageBytes);
-    uint64_t* empty = full + kUStages;
-    uint64_t* done = empty + kUStages;
+    uint64_t* full = reinterpret_cast<uint64_t*>(sm + U::ST * U::stage_bytes);
+    uint64_t* empty = full + U::ST;
+    uint64_t* done = empty + U::ST;
     uint64_t* sum_full = done + 1;    // a chain of the high parts' products is complete
     uint64_t* sum_empty = done + 2;   // it has been read
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 3);
@@ -129,7 +134,7 @@ __global__ void __launch_bounds__(U::threads, 1)
     volatile int* everr = err;
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < kUStages; ++i) {
+        for (int i = 0; i < U::ST; ++i) {
             u_mb_init(&full[i], 1);
             u_mb_init(&empty[i], 1);
         }
@@ -140,7 +145,7 @@ __global__ void __launch_bounds__(U::threads, 1)
     }
     if (w == U::EW) {  // tensor memory for the accumulators
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(u_saddr(tmem_slot)),
-                     "r"(kUTmemCols)
+                     "r"(U::tmem_cols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -151,11 +156,11 @@ __global__ void __launch_bounds__(U::threads, 1)
     // The weights do not depend on the previous kernel: the first stages'
     // weight blocks are requested before the programmatic wait, so that
     // their HBM latency overlaps the previous kernel's tail.
-    const int pre = ks < kUStages ? ks : kUStages;
+    const int pre = ks < U::ST ? ks : U::ST;
     if (w == U::EW && lane == 0)
         for (int i = 0; i < pre; ++i) {
             u_expect_tx(&full[i], stage_tx);
-            u_tma_w(sm + i * kUStageBytes, &wmap, tile0, (k0 + i) * (kUKStage / 8), &full[i]);
+            u_tma_w(sm + i * U::stage_bytes, &wmap, tile0, (k0 + i) * (kUKStage / 8), &full[i]);
         }
     // the set-up above overlaps the previous kernel (programmatic launch)
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -166,13 +171,13 @@ __global__ void __launch_bounds__(U::threads, 1)
         int issued = 0;
         bool ok = true;
         for (int i = 0; i < ks && ok; ++i) {
-            const int st = i % kUStages;
-            if (i >= kUStages && !u_mb_wait(&empty[st], ((i / kUStages) - 1) & 1, everr)) {
+            const int st = i % U::ST;
+            if (i >= U::ST && !u_mb_wait(&empty[st], ((i / U::ST) - 1) & 1, everr)) {
                 atomicOr(err, kErrStall);
                 ok = false;
                 break;
             }
-            uint8_t* a = sm + st * kUStageBytes;
+            uint8_t* a = sm + st * U::stage_bytes;
             const int kc = (k0 + i) * (kUKStage / 8);  // first 16-byte chunk of the stage
             if (i >= pre) {  // (the first stages' weights are in flight already)
                 u_expect_tx(&full[st], stage_tx);
@@ -183,8 +188,8 @@ __global__ void __launch_bounds__(U::threads, 1)
             ++issued;
         }
         // every issued copy lands before the CTA may leave
-        for (int i = issued > kUStages ? issued - kUStages : 0; i < issued; ++i)
-            u_mb_wait(&full[i % kUStages], (i / kUStages) & 1, nullptr);
+        for (int i = issued > U::ST ? issued - U::ST : 0; i < issued; ++i)
+            u_mb_wait(&full[i % U::ST], (i / U::ST) & 1, nullptr);
     } else if (w == U::EW + 1 && lane == 0) {
         // MMA issuer
         const uint32_t idesc = u_idesc(N);
@@ -196,11 +201,11 @@ __global__ void __launch_bounds__(U::threads, 1)
         const uint64_t da0 = u_desc(a0, 2048, 128), db0 = u_desc(a0 + kUABytes, 3 * part_bytes, 128);
         const uint32_t part16 = part_bytes >> 4;
         auto mma = [&](int st, int kk, int pp, bool fresh) {
-            const uint32_t at = st * (kUStageBytes >> 4);
-            u_mma(tmem + (pp ? kRowsBlock : 0), da0 + (at + kk * 256), db0 + (at + (kk * 6 + pp) * part16), idesc, fresh ? 0u : 1u);
+            const uint32_t at = st * (U::stage_bytes >> 4);
+            u_mma(tmem + (pp ? U::rows : 0), da0 + (at + kk * 256), db0 + (at + (kk * 6 + pp) * part16), idesc, fresh ? 0u : 1u);
         };
         auto landed = [&](int i) {
-            const bool ok = u_mb_wait(&full[i % kUStages], (i / kUStages) & 1, everr);
+            const bool ok = u_mb_wait(&full[i % U::ST], (i / U::ST) & 1, everr);
             if (!ok) atomicOr(err, kErrStall);
             u_fence_after();
             return ok;
@@ -217,8 +222,8 @@ __global__ void __launch_bounds__(U::threads, 1)
                     ok = landed(i + k);
 #pragma unroll
                     for (int kk = 0; kk < kUKStage / 16 && ok; ++kk) {
-                        mma((i + k) % kUStages, kk, 1, false);
-                        mma((i + k) % kUStages, kk, 2, false);
+                        mma((i + k) % U::ST, kk, 1, false);
+                        mma((i + k) % U::ST, kk, 2, false);
                     }
                 }
                 if (ok && !u_mb_wait(sum_empty, (i / U::CH - 1) & 1, everr)) {
@@ -229,8 +234,8 @@ __global__ void __launch_bounds__(U::threads, 1)
                 u_fence_after();
                 for (int k = 0; k < n; ++k) {
 #pragma unroll
-                    for (int kk = 0; kk < kUKStage / 16; ++kk) mma((i + k) % kUStages, kk, 0, k == 0 && kk == 0);
-                    u_commit(&empty[(i + k) % kUStages]);
+                    for (int kk = 0; kk < kUKStage / 16; ++kk) mma((i + k) % U::ST, kk, 0, k == 0 && kk == 0);
+                    u_commit(&empty[(i + k) % U::ST]);
                 }
                 i += n;
             } else {
@@ -239,8 +244,8 @@ __global__ void __launch_bounds__(U::threads, 1)
 #pragma unroll
                 for (int kk = 0; kk < kUKStage / 16; ++kk)
 #pragma unroll
-                    for (int pp = 0; pp < 3; ++pp) mma(i % kUStages, kk, pp, i == 0 && kk == 0 && pp < 2);
-                u_commit(&empty[i % kUStages]);
+                    for (int pp = 0; pp < 3; ++pp) mma(i % U::ST, kk, pp, i == 0 && kk == 0 && pp < 2);
+                u_commit(&empty[i % U::ST]);
                 ++i;
             }
         }
@@ -292,7 +297,7 @@ __global__ void __launch_bounds__(U::threads, 1)
                 if (col0 + c < M) {
                     float hi[16], ml[16];
                     u_ld16(lane_addr + c, hi);
-                    u_ld16(lane_addr + kRowsBlock + c, ml);
+                    u_ld16(lane_addr + U::rows + c, ml);
                     if (tile < n_tiles)
 #pragma unroll
                         for (int i = 0; i < 16; ++i)
@@ -302,7 +307,7 @@ __global__ void __launch_bounds__(U::threads, 1)
     }
     u_fence_before();
     __syncthreads();
-    if (w == U::EW) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kUTmemCols) : "memory");
+    if (w == U::EW) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(U::tmem_cols) : "memory");
 }
 
 // ---------------------------------------------------------------- host side
@@ -338,8 +343,7 @@ bool weight_map(CUtensorMap* map, const uint16_t* W, int64_t n_tiles, int K) {
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-bool small_batch(int M) { return x3_rows(M) <= USmall::EW / 4 * USmall::HC; }
-size_t umma_smem() { return (size_t)kUStages * kUStageBytes + 256 + 1024; }
+bool small_batch(int M) { return x3_rows(M) <= USmall::rows; }
 
 }  // namespace
 
@@ -353,9 +357,9 @@ bool umma_available() {
         CUtensorMap probe;
         static uint16_t dummy[64 * 8] __attribute__((aligned(16)));
         ok = major == 10 && encode_fn() && weight_map(&probe, dummy, 4, 64) &&
-             cudaFuncSetAttribute(k_rows_umma<ULarge>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)umma_smem()) ==
+             cudaFuncSetAttribute(k_rows_umma<ULarge>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ULarge::smem) ==
                  cudaSuccess &&
-             cudaFuncSetAttribute(k_rows_umma<USmall>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)umma_smem()) ==
+             cudaFuncSetAttribute(k_rows_umma<USmall>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)USmall::smem) ==
                  cudaSuccess &&
              configure_uattn() == cudaSuccess;
         cudaGetLastError();
@@ -369,8 +373,9 @@ bool umma_available() {
 // every CTA's run of stages and lengthens the sum that the next launch starts
 // with, each by about the same time, so there are at most sqrt(2 stages) of
 // them.  A 33-position prompt at 0.5B (21 splits of two stages or fewer became
-// 7 of four, 21 of seven became 17 of nine): 1300 us before, 1254 now; 1262 with
-// sqrt(stages) splits, 1263 with sqrt(4 stages).
+// 7 of four, 21 of seven became 17 of nine): 1300 us before, 1254 with it
+// (1244 since USmall has eight stages); 1262 with sqrt(stages) splits, 1263 with
+// sqrt(4 stages).
 int umma_splits(int64_t n_tiles, int K, int M, int n_sm) {
     const int64_t mt = (n_tiles + 3) / 4 * rows_blocks(M);
     const int nk = (K + kUKStage - 1) / kUKStage;
@@ -390,7 +395,7 @@ cudaError_t launch_mm_umma(const uint16_t* W, int64_t n_rows, int K, const uint1
     cfg.gridDim = grid;
     const bool small = small_batch(M);
     cfg.blockDim = dim3(small ? USmall::threads : ULarge::threads);
-    cfg.dynamicSmemBytes = umma_smem();
+    cfg.dynamicSmemBytes = small ? USmall::smem : ULarge::smem;
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
