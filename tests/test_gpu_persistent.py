@@ -103,6 +103,34 @@ def test_1p5b_persistent_agrees_with_five_launch_path():
     assert np.max(np.abs(c0[:first_diff] - c1[:first_diff]), initial=0) < 1e-3
 
 
+def test_ring_products_round_like_short_chains():
+    """Rounding of the ring-fed products (LM head of a 2048-wide model) against
+    64 bits, the scale that all logits share taken out.  A rounding to nearest
+    of x errs by 0.18 (2^-24 x)^2 in the mean square; counted over the partial
+    sums of random terms, a row of 2048 summed stage by stage (8 terms, 4
+    stages, 2 halves, 4 column groups, 8 warps) comes to 1.70 2^-24 of the
+    logits, the input's two roundings included, and one chain of 32 terms per
+    half to 2.15 2^-24.  4096 logits scatter by 2%."""
+    from paper_2609_14144_gb300 import OPT_DEBUG_LOGITS, Engine
+
+    shape = TINY.replace(d_model=2048, n_layers=1, readout_layers=(1,))
+    model = synth.make_model(shape)
+    eng = Engine(shape, model)
+    assert eng.persistent
+    eng.set_option(OPT_DEBUG_LOGITS, 1)
+    eng.prefill(synth.prompt(shape, 3))
+    off = []
+    for tok in range(4):
+        eng.decode_step(tok, [2.0], oracle.FORCE_FULL)
+        h = eng.hidden_final().astype(np.float64)
+        z = h / np.sqrt((h * h).mean() + np.float32(shape.rms_eps)) * synth.bf16_to_f32(model["final_norm"])
+        ref = synth.bf16_to_f32(model["lm_head"]).astype(np.float64) @ z
+        e = eng.final_logits() - ref
+        e -= ref * (e @ ref) / (ref @ ref)
+        off.append(np.sqrt((e @ e) / (ref @ ref)) * 2.0 ** 24)
+    assert np.mean(off) <= 1.9, off
+
+
 def test_waits_that_run_out_report_a_stall_and_reset_recovers():
     """Failure detection of the persistent layer kernel's bounded waits: with
     the wait bound lowered to 400 SM cycles, ordinary waits (ring stages,
