@@ -298,8 +298,8 @@ cudaError_t rows_pass(const DevModel& m, const RowsBuf& b, const int* start, int
 // the warp-level path).
 bool umma_available();
 int umma_splits(int64_t n_tiles, int K, int M, int n_sm);
-cudaError_t launch_mm_umma(const uint16_t* W, int64_t n_rows, int K, const uint16_t* x3, int ldx, int M, int S, float* part,
-                           int Np, int* err, cudaStream_t s);
+cudaError_t launch_mm_umma(const uint16_t* W, int64_t n_rows, int K, const uint16_t* x3, int ldx, int M, int S, int n_sm,
+                           float* part, int Np, int* err, cudaStream_t s);
 // tcgen05 attention of a batch (ee_uattn.cu), for batches of at least
 // kUaMinRows rows: keys per split, the launch (its split outputs in the
 // warp-level kernel's layout).

@@ -824,7 +824,7 @@ cudaError_t launch_mm(const uint16_t* W, int64_t n_rows, int K, const RowsBuf& b
         Np = (int)(nt * kTileRows);
         S = umma_splits(nt, K, M, b.n_sm);
         S = (int)std::max<int64_t>(1, std::min<int64_t>(S, b.part_floats / ((int64_t)M * Np)));
-        return launch_mm_umma(W, n_rows, K, b.x3, b.ldx, M, S, b.part, Np, b.err, s);
+        return launch_mm_umma(W, n_rows, K, b.x3, b.ldx, M, S, b.n_sm, b.part, Np, b.err, s);
     }
     int NB, RG;
     row_groups(M, NB, RG);

@@ -38,8 +38,10 @@
 // number of steps it is carried through: with a whole K range in one chain a
 // 4099-position prompt was 2.0e-4 from 64 bits in its final state, with chains
 // of 4 stages 2.5e-5.  Reading a chain back costs little tensor time: the next
-// two stages' middle and low parts' products are issued first and run under it
-// (gate/up of an 820-row batch at 3B: 162 us, 145 us in one chain).
+// stages' middle and low parts' products are issued first and run under it
+// (gate/up of an 820-row batch at 3B: 162 us, 145 us in one chain).  A chain is
+// never longer than a split of a 256-row batch (umma_chain): where K is short
+// and the splits are many there, fewer splits must not mean longer chains.
 // Every wait is bounded; after a wait runs out the kernel flags kErrStall in
 // the device error word, waits (bounded, whatever the word says) for its
 // copies in flight and for the MMAs it issued, frees its tensor memory and
@@ -64,26 +66,30 @@ constexpr int kUABytes = kUMRows * kUKStage * 2;    // 8 KB
 
 // A launch's shape.  EW epilogue warps read the accumulators (warp w:
 // tensor-memory lanes 32 (w mod 4), columns from HC (w / 4) on), then come the
-// producer warp and the MMA warp; CH stages of the high parts' products (at
-// most) add up in tensor memory.
-template <int EW_, int HC_, int CH_, int ST_>
+// producer warp and the MMA warp; NA accumulators of the high parts' products,
+// CH stages to a chain (0: as many as the launch says).
+template <int EW_, int HC_, int NA_, int CH_, int ST_>
 struct UShape {
-    static constexpr int EW = EW_, HC = HC_, CH = CH_, ST = ST_;
+    static constexpr int EW = EW_, HC = HC_, NA = NA_, CH = CH_, ST = ST_;
     static constexpr int threads = 32 * (EW + 2);
     static constexpr int rows = EW / 4 * HC;  // a block's rows, at most
     // a stage: the weight block and the activations of a full block (8 + 48, 8 + 12 KB)
     static constexpr int stage_bytes = kUABytes + kUKStage / 8 * 3 * rows * 16;
-    static constexpr int tmem_cols = 2 * rows;  // two accumulators of one fp32 column per position
+    static constexpr int lo = NA * rows;      // the middle and low parts' accumulator
+    static constexpr int tmem_cols = 512;     // accumulators of one fp32 column per position (a CTA has the SM to itself)
     static constexpr size_t smem = (size_t)ST * stage_bytes + 256 + 1024;
+    static_assert(lo + rows <= tmem_cols, "the accumulators fit tensor memory");
 };
-using ULarge = UShape<8, kRowsBlock / 2, 4, 4>;
+using ULarge = UShape<8, kRowsBlock / 2, 1, 4, 4>;
+using UShort = UShape<8, kRowsBlock / 2, 1, 0, 4>;  // short K ranges: shorter chains
 // A small batch: fewer threads and registers, so that the launches before and
-// after find room beside it (programmatic launch), and longer chains, since its
-// products are too short to run under a read-back.  Eight of its small stages,
+// after find room beside it (programmatic launch).  Its products are too short
+// to run under a read-back, but its accumulators are narrow: each chain has one
+// of its own, all read after the last stage.  Eight of its small stages,
 // so that most splits have their whole range in flight at once, the weights
 // since before the programmatic wait (33 positions at 0.5B: 1254 us with four
 // stages as long as a full block's, 1267 with four short ones, 1244 with eight).
-using USmall = UShape<4, 64, 24, 8>;
+using USmall = UShape<4, 64, 4, 0, 8>;
 
 // ---------------------------------------------------------------- copies
 __device__ __forceinline__ void u_expect_tx(uint64_t* bar, uint32_t bytes) {
@@ -109,7 +115,8 @@ __device__ __forceinline__ void u_bulk(void* dst, const void* src, uint32_t byte
 template <class U>
 __global__ void __launch_bounds__(U::threads, 1)
     k_rows_umma(const __grid_constant__ CUtensorMap wmap, const uint16_t* __restrict__ x3, int ldx, int n_tiles, int K,
-                int M_all, int S, float* __restrict__ part, int Np, int* err) {
+                int M_all, int S, int chain, float* __restrict__ part, int Np, int* err) {
+    const int ch = U::CH ? U::CH : chain;
     extern __shared__ __align__(1024) uint8_t u_smem_raw[];
     uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(u_smem_raw) + 1023) & ~(uintptr_t)1023);
     uint64_t* full = reinterpret_cast<uint64_t*>(sm + U::ST * U::stage_bytes);
@@ -200,9 +207,9 @@ __global__ void __launch_bounds__(U::threads, 1)
         const uint32_t a0 = u_saddr(sm);
         const uint64_t da0 = u_desc(a0, 2048, 128), db0 = u_desc(a0 + kUABytes, 3 * part_bytes, 128);
         const uint32_t part16 = part_bytes >> 4;
-        auto mma = [&](int st, int kk, int pp, bool fresh) {
+        auto mma = [&](int st, int kk, int pp, int acc, bool fresh) {
             const uint32_t at = st * (U::stage_bytes >> 4);
-            u_mma(tmem + (pp ? U::rows : 0), da0 + (at + kk * 256), db0 + (at + (kk * 6 + pp) * part16), idesc, fresh ? 0u : 1u);
+            u_mma(tmem + (pp ? U::lo : acc * U::rows), da0 + (at + kk * 256), db0 + (at + (kk * 6 + pp) * part16), idesc, fresh ? 0u : 1u);
         };
         auto landed = [&](int i) {
             const bool ok = u_mb_wait(&full[i % U::ST], (i / U::ST) & 1, everr);
@@ -211,43 +218,51 @@ __global__ void __launch_bounds__(U::threads, 1)
             return ok;
         };
         bool ok = true;
+        int since = 0, q = 0;  // stages of the chain so far; the chain
         for (int i = 0; i < ks && ok;) {
-            if (i > 0 && i % U::CH == 0) {
-                // The high parts start a new chain: two stages' middle and low
-                // parts' products first, which run while the epilogue warps
-                // read the old one.
-                u_commit(sum_full);
-                const int n = ks - i < 2 ? 1 : 2;
-                for (int k = 0; k < n && ok; ++k) {
-                    ok = landed(i + k);
+            if (since == ch) {
+                since = 0;
+                ++q;
+                if constexpr (U::NA == 1) {
+                    // The high parts start a new chain in the one accumulator:
+                    // two stages' middle and low parts' products first, which
+                    // run while the epilogue warps read the old chain.
+                    u_commit(sum_full);
+                    const int n = min(ks - i, min(ch, 2));
+                    for (int k = 0; k < n && ok; ++k) {
+                        ok = landed(i + k);
 #pragma unroll
-                    for (int kk = 0; kk < kUKStage / 16 && ok; ++kk) {
-                        mma((i + k) % U::ST, kk, 1, false);
-                        mma((i + k) % U::ST, kk, 2, false);
+                        for (int kk = 0; kk < kUKStage / 16 && ok; ++kk) {
+                            mma((i + k) % U::ST, kk, 1, 0, false);
+                            mma((i + k) % U::ST, kk, 2, 0, false);
+                        }
                     }
-                }
-                if (ok && !u_mb_wait(sum_empty, (i / U::CH - 1) & 1, everr)) {
-                    atomicOr(err, kErrStall);
-                    ok = false;
-                }
-                if (!ok) break;
-                u_fence_after();
-                for (int k = 0; k < n; ++k) {
+                    if (ok && !u_mb_wait(sum_empty, (q - 1) & 1, everr)) {
+                        atomicOr(err, kErrStall);
+                        ok = false;
+                    }
+                    if (!ok) break;
+                    u_fence_after();
+                    for (int k = 0; k < n; ++k) {
 #pragma unroll
-                    for (int kk = 0; kk < kUKStage / 16; ++kk) mma((i + k) % U::ST, kk, 0, k == 0 && kk == 0);
-                    u_commit(&empty[(i + k) % U::ST]);
+                        for (int kk = 0; kk < kUKStage / 16; ++kk) mma((i + k) % U::ST, kk, 0, 0, k == 0 && kk == 0);
+                        u_commit(&empty[(i + k) % U::ST]);
+                    }
+                    i += n;
+                    since = n;
+                    continue;
                 }
-                i += n;
-            } else {
-                ok = landed(i);
-                if (!ok) break;
-#pragma unroll
-                for (int kk = 0; kk < kUKStage / 16; ++kk)
-#pragma unroll
-                    for (int pp = 0; pp < 3; ++pp) mma(i % U::ST, kk, pp, i == 0 && kk == 0 && pp < 2);
-                u_commit(&empty[i % U::ST]);
-                ++i;
             }
+            ok = landed(i);
+            if (!ok) break;
+#pragma unroll
+            for (int kk = 0; kk < kUKStage / 16; ++kk)
+#pragma unroll
+                for (int pp = 0; pp < 3; ++pp)
+                    mma(i % U::ST, kk, pp, U::NA == 1 ? 0 : q, kk == 0 && (pp ? i == 0 && pp == 1 : since == 0));
+            u_commit(&empty[i % U::ST]);
+            ++i;
+            ++since;
         }
         u_commit(done);  // after every MMA this thread issued
     }
@@ -258,32 +273,34 @@ __global__ void __launch_bounds__(U::threads, 1)
         constexpr int HC = U::HC;
         const int col0 = (w >> 2) * HC, tile = tile0 + (w & 3);
         const uint32_t lane_addr = tmem + ((uint32_t)(32 * (w & 3)) << 16) + col0;
-        float sum[HC];
+        float sum[U::NA == 1 ? HC : 1];
+        if constexpr (U::NA == 1) {
 #pragma unroll
-        for (int i = 0; i < HC; ++i) sum[i] = 0.f;
-        for (int f = 0; f < (ks - 1) / U::CH; ++f) {
-            if (!u_mb_wait(sum_full, f & 1, everr)) {
-                atomicOr(err, kErrStall);
-                break;
-            }
-            u_fence_after();
-            __syncwarp();
-#pragma unroll
-            for (int c = 0; c < HC; c += 32)
-                if (col0 + c < M) {
-                    uint32_t v0[16], v1[16];
-                    u_ld16(lane_addr + c, v0);
-                    u_ld16(lane_addr + c + 16, v1);
-                    u_wait_ld();
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        sum[c + i] += __uint_as_float(v0[i]);
-                        sum[c + 16 + i] += __uint_as_float(v1[i]);
-                    }
+            for (int i = 0; i < HC; ++i) sum[i] = 0.f;
+            for (int f = 0; f < (ks - 1) / ch; ++f) {
+                if (!u_mb_wait(sum_full, f & 1, everr)) {
+                    atomicOr(err, kErrStall);
+                    break;
                 }
-            u_fence_before();
-            __syncwarp();
-            if (lane == 0) u_mb_arrive(sum_empty);
+                u_fence_after();
+                __syncwarp();
+#pragma unroll
+                for (int c = 0; c < HC; c += 32)
+                    if (col0 + c < M) {
+                        uint32_t v0[16], v1[16];
+                        u_ld16(lane_addr + c, v0);
+                        u_ld16(lane_addr + c + 16, v1);
+                        u_wait_ld();
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) {
+                            sum[c + i] += __uint_as_float(v0[i]);
+                            sum[c + 16 + i] += __uint_as_float(v1[i]);
+                        }
+                    }
+                u_fence_before();
+                __syncwarp();
+                if (lane == 0) u_mb_arrive(sum_empty);
+            }
         }
         bool have = u_mb_wait(done, 0, nullptr);  // the MMA thread commits done after every wait of its own
         if (!have) have = u_mb_wait(done, 0, nullptr);
@@ -295,13 +312,34 @@ __global__ void __launch_bounds__(U::threads, 1)
 #pragma unroll
             for (int c = 0; c < HC; c += 16)
                 if (col0 + c < M) {
-                    float hi[16], ml[16];
-                    u_ld16(lane_addr + c, hi);
-                    u_ld16(lane_addr + U::rows + c, ml);
+                    float t[16];
+                    if constexpr (U::NA == 1) {
+                        uint32_t hi[16], lo[16];
+                        u_ld16(lane_addr + c, hi);
+                        u_wait_ld();
+                        u_ld16(lane_addr + U::lo + c, lo);
+                        u_wait_ld();
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) t[i] = sum[c + i] + (__uint_as_float(hi[i]) + __uint_as_float(lo[i]));
+                    } else {  // the chains that there are, then the middle and low parts
+                        uint32_t v[U::NA + 1][16];
+#pragma unroll
+                        for (int k = 0; k < U::NA; ++k)
+                            if (k * ch < ks) u_ld16(lane_addr + k * U::rows + c, v[k]);
+                        u_ld16(lane_addr + U::lo + c, v[U::NA]);
+                        u_wait_ld();
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) t[i] = __uint_as_float(v[U::NA][i]);
+#pragma unroll
+                        for (int k = 0; k < U::NA; ++k)
+                            if (k * ch < ks)
+#pragma unroll
+                                for (int i = 0; i < 16; ++i) t[i] += __uint_as_float(v[k][i]);
+                    }
                     if (tile < n_tiles)
 #pragma unroll
                         for (int i = 0; i < 16; ++i)
-                            if (col0 + c + i < M) ps[(int64_t)(c + i) * Np + n] = sum[c + i] + (hi[i] + ml[i]);
+                            if (col0 + c + i < M) ps[(int64_t)(c + i) * Np + n] = t[i];
                 }
         }
     }
@@ -359,6 +397,8 @@ bool umma_available() {
         ok = major == 10 && encode_fn() && weight_map(&probe, dummy, 4, 64) &&
              cudaFuncSetAttribute(k_rows_umma<ULarge>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ULarge::smem) ==
                  cudaSuccess &&
+             cudaFuncSetAttribute(k_rows_umma<UShort>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)UShort::smem) ==
+                 cudaSuccess &&
              cudaFuncSetAttribute(k_rows_umma<USmall>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)USmall::smem) ==
                  cudaSuccess &&
              configure_uattn() == cudaSuccess;
@@ -385,8 +425,20 @@ int umma_splits(int64_t n_tiles, int K, int M, int n_sm) {
     return (int)std::max<int64_t>(1, want);
 }
 
-cudaError_t launch_mm_umma(const uint16_t* W, int64_t n_rows, int K, const uint16_t* x3, int ldx, int M, int S, float* part,
-                           int Np, int* err, cudaStream_t s) {
+// Stages per chain.  A small batch: an accumulator for each.  A full block: 4,
+// fewer where a split of a 256-row batch (one CTA per SM)
+// would be shorter, so that short K ranges are summed no less exactly when
+// larger batches leave them fewer splits (feed-forward of 1000 rows at width 256:
+// error 3.4e-7 with chains of 4, 1.8e-7 in splits of one stage).
+static int umma_chain(int64_t n_tiles, int K, int M, int S, int n_sm) {
+    const int nk = (K + kUKStage - 1) / kUKStage;
+    if (small_batch(M)) return ((nk + S - 1) / S + USmall::NA - 1) / USmall::NA;
+    const int64_t splits = std::max<int64_t>(1, n_sm / ((n_tiles + 3) / 4));
+    return (int)std::max<int64_t>(1, std::min<int64_t>(ULarge::CH, nk / splits));
+}
+
+cudaError_t launch_mm_umma(const uint16_t* W, int64_t n_rows, int K, const uint16_t* x3, int ldx, int M, int S, int n_sm,
+                           float* part, int Np, int* err, cudaStream_t s) {
     const int64_t nt = tile_count(n_rows);
     CUtensorMap map;
     if (!weight_map(&map, W, nt, K)) return cudaErrorNotSupported;
@@ -394,6 +446,7 @@ cudaError_t launch_mm_umma(const uint16_t* W, int64_t n_rows, int K, const uint1
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     const bool small = small_batch(M);
+    const int ch = umma_chain(nt, K, M, S, n_sm);
     cfg.blockDim = dim3(small ? USmall::threads : ULarge::threads);
     cfg.dynamicSmemBytes = small ? USmall::smem : ULarge::smem;
     cfg.stream = s;
@@ -402,8 +455,9 @@ cudaError_t launch_mm_umma(const uint16_t* W, int64_t n_rows, int K, const uint1
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    if (small) return cudaLaunchKernelEx(&cfg, k_rows_umma<USmall>, map, x3, ldx, (int)nt, K, M, S, part, Np, err);
-    return cudaLaunchKernelEx(&cfg, k_rows_umma<ULarge>, map, x3, ldx, (int)nt, K, M, S, part, Np, err);
+    if (small) return cudaLaunchKernelEx(&cfg, k_rows_umma<USmall>, map, x3, ldx, (int)nt, K, M, S, ch, part, Np, err);
+    if (ch < ULarge::CH) return cudaLaunchKernelEx(&cfg, k_rows_umma<UShort>, map, x3, ldx, (int)nt, K, M, S, ch, part, Np, err);
+    return cudaLaunchKernelEx(&cfg, k_rows_umma<ULarge>, map, x3, ldx, (int)nt, K, M, S, ch, part, Np, err);
 }
 
 }  // namespace ee

@@ -88,13 +88,6 @@ __device__ __forceinline__ void u_ld16(uint32_t taddr, uint32_t (&r)[16]) {
         : "memory");
 }
 __device__ __forceinline__ void u_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void u_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    u_ld16(taddr, r);
-    u_wait_ld();
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
 
 }  // namespace ee
 

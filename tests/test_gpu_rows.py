@@ -14,7 +14,7 @@ import pytest
 
 import oracle
 import synth
-from helpers import EXCLUDE_EPS, REL_TOL, check_kv, rel_err
+from helpers import EXCLUDE_EPS, REL_TOL, bf16_bits_to_f32, check_kv, rel_err, to_bf16_bits
 
 pytestmark = pytest.mark.gpu
 
@@ -140,6 +140,35 @@ def test_tcgen05_attention_row_and_key_edges(n, D, page):
         if 0 <= t < n:  # layer 1's entries carry layer 0's attention of that row
             for x, y in zip(a.kv(1, t), b.kv(1, t)):
                 assert rel_err(x, y) <= REL_TOL, t
+
+
+@pytest.mark.parametrize("n", [48, 64, 400, 1000])
+def test_batched_products_round_like_short_chains(n):
+    """The feed-forward of one layer (width 256: 8 and 22 stages of 32 columns
+    in all) for a prompt's last row, against 64 bits.  The tensor core drops
+    what an addition shifts out: half a unit in the last place on average, and
+    always towards zero, so it adds up over a chain of additions.  With chains
+    of one stage (two additions) the three products come to about 1.6e-7, with
+    two or more stages to 2.5e-7 and 3.4e-7; 16 rows scatter by a tenth."""
+    shape = TINY.replace(n_layers=2, readout_layers=(1,))
+    model = synth.make_model(shape)
+    for j, lw in enumerate(model["layers"]):  # layer 0 is its feed-forward alone, layer 1 adds nothing
+        lw["wo"] = np.zeros_like(lw["wo"])
+        lw["wd"] = to_bf16_bits(bf16_bits_to_f32(lw["wd"]) * (20 if j == 0 else 0))
+    w = {k: synth.bf16_to_f32(v).astype(np.float64) for k, v in model["layers"][0].items()}
+    embed = synth.bf16_to_f32(model["embed"]).astype(np.float64)
+    eng = _engine(shape, model, n + 1)
+    off = []
+    for i in range(16):
+        prompt = synth.token_ids(shape.seed, 920 + i, n, shape.vocab)
+        eng.reset()
+        eng.prefill(prompt)
+        x = embed[prompt[-1]]
+        z = x / np.sqrt((x * x).mean() + np.float32(shape.rms_eps)) * w["mlp_norm"]
+        g = w["wg"] @ z
+        ref = w["wd"] @ (g / (1 + np.exp(-g)) * (w["wu"] @ z))
+        off.append(np.linalg.norm(eng.hidden_final() - x - ref) / np.linalg.norm(ref))
+    assert np.exp(np.mean(np.log(off))) <= 2.1e-7, off
 
 
 def _exit_decode(shape, model, n, force_of, rows=True):
