@@ -80,6 +80,35 @@ def test_attention_decode_groups_tiles_and_pages(T, P, D, G):
     assert err <= 4.5 * math.sqrt(T) * 2.0 ** -24 * 8, err
 
 
+@pytest.mark.parametrize("T,most", [(17, 1.31e-7), (100, 1.63e-7)])
+def test_attention_decode_rounds_like_short_chains(T, most):
+    """The mean error of short calls against 64 bits.  A rounding to nearest of
+    x errs by 0.18 (2^-24 x)^2 in the mean square; counted over the partial sums
+    of a score of 128 dimensions (chunks of 8, four chunks, four lanes) that is
+    7.5e-8, which each probability and so the output takes over; the rest
+    (queries scaled, exponentials, sums over positions) is 9.2e-8 at 17
+    positions and 1.2e-7 at 100.  Together 1.19e-7 and 1.47e-7; with one chain
+    of 32 dimensions a lane 1.45e-7 and 1.8e-7."""
+    import torch
+
+    from paper_2609_14144_gb300 import attention_decode
+
+    A, KH, D, P = 16, 2, 128, 64
+    off = []
+    for seed in range(32):
+        g = torch.Generator(device="cuda").manual_seed(seed)
+        n_pages = (T + P - 1) // P
+        q = torch.randn(A * D, generator=g, device="cuda")
+        kp = torch.randn(n_pages, KH, P, D, generator=g, device="cuda").to(torch.bfloat16)
+        vp = torch.randn(n_pages, KH, P, D, generator=g, device="cuda").to(torch.bfloat16)
+        table = torch.arange(n_pages, device="cuda", dtype=torch.int32)
+        k, v = (t.double().permute(1, 0, 2, 3).reshape(KH, -1, D)[:, :T] for t in (kp, vp))
+        ref = torch.softmax(q.double().view(KH, A // KH, D) @ k.transpose(1, 2) / math.sqrt(D), -1) @ v
+        got = attention_decode(q, kp, vp, table, T, A, KH, D, P).view_as(ref)
+        off.append(((got - ref).norm() / ref.norm()).item())
+    assert np.exp(np.mean(np.log(off))) <= most, off
+
+
 @pytest.mark.parametrize("V,d", [(4096, 256), (4093, 256), (151936, 896), (151937, 1536), (1000, 2048)])
 def test_vocab_confidence(V, d):
     import torch
