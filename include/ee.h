@@ -388,7 +388,9 @@ int ee_attention_decode_static(const float* q, const uint16_t* k_pages, const ui
  *   out_token device int32[1] (lowest argmax), out_p device float[1]
  *   logits   device fp32 [V] or NULL
  *   scratch  device workspace of ee_vocab_scratch_bytes() bytes
- * Enqueued on stream. */
+ * Enqueued on stream.  The kernel's waits for its own copies are bounded (about
+ * 2 s); should one run out, out_token is -1, out_p (the signals) NaN, and so are
+ * the logits it could not compute. */
 int ee_vocab_scratch_bytes(int vocab, int d_model, size_t* bytes);
 int ee_vocab_confidence(const float* x, const uint16_t* gain, const uint16_t* U, int vocab, int d_model,
                         float eps, void* scratch, size_t scratch_bytes, int32_t* out_token, float* out_p,

@@ -1513,7 +1513,7 @@ int ee_vocab_scratch_bytes(int vocab, int d_model, size_t* bytes) {
 namespace {
 int vocab_standalone(const float* x, const uint16_t* gain, const uint16_t* U, int vocab, int d_model, float eps,
                      void* scratch, size_t scratch_bytes, int32_t* out_token, float* out_p, float* out_sig,
-                     float* logits, void* stream) {
+                     float* logits, void* stream, long long wait_cycles = 0) {
     size_t need = 0;
     EE_TRY(ee_vocab_scratch_bytes(vocab, d_model, &need));
     if (!x || !gain || !U || !scratch || !out_token || (!out_p && !out_sig)) return fail(EE_EINVAL, "NULL argument");
@@ -1544,7 +1544,8 @@ int vocab_standalone(const float* x, const uint16_t* gain, const uint16_t* U, in
     // the ring wants 16-byte rows on 16-byte boundaries (the d_model % 8 that
     // ee_vocab_scratch_bytes checks) and the row's columns in registers
     if (d_model <= kVocabRowsMaxD)
-        EE_CK(launch_vocab_rows(v, std::min(nsm, kMaxVocabCtas), s));
+        EE_CK(launch_vocab_rows(v, std::min(nsm, kMaxVocabCtas), wait_cycles ? wait_cycles : kSegStallCycles,
+                                wait_cycles ? std::max(1LL, wait_cycles / 4) : kSegCheckCycles, s));
     else
         EE_CK(launch_vocab(v, std::min(nsm, kMaxVocabCtas), false, s));
     return EE_OK;
@@ -1565,6 +1566,16 @@ int ee_vocab_signals(const float* x, const uint16_t* gain, const uint16_t* U, in
     if (!out_signals) return fail(EE_EINVAL, "NULL argument");
     return vocab_standalone(x, gain, U, vocab, d_model, eps, scratch, scratch_bytes, out_token, nullptr,
                             out_signals, logits, stream);
+}
+
+// For the tests of failure detection, not in ee.h: ee_vocab_signals with the
+// bound of the kernel's waits lowered to wait_cycles SM cycles.
+int ee_vocab_signals_bounded(const float* x, const uint16_t* gain, const uint16_t* U, int vocab, int d_model, float eps,
+                             void* scratch, size_t scratch_bytes, int32_t* out_token, float* out_signals, float* logits,
+                             void* stream, long long wait_cycles) {
+    if (!out_signals || wait_cycles <= 0) return fail(EE_EINVAL, "bad argument");
+    return vocab_standalone(x, gain, U, vocab, d_model, eps, scratch, scratch_bytes, out_token, nullptr,
+                            out_signals, logits, stream, wait_cycles);
 }
 
 int ee_select_tau(const float* conf, int conf_stride, const int32_t* member, int n, float target, float* tau,

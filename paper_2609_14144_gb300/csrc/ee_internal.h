@@ -170,7 +170,9 @@ cudaError_t launch_vocab(const VocabArgs& v, int grid, bool pdl, cudaStream_t s)
 // The pass over a caller's row-major U fed through a shared-memory ring
 // (ee_persist.cu): one CTA per SM; rows of up to kVocabRowsMaxD columns.
 constexpr int kVocabRowsMaxD = 2048;
-cudaError_t launch_vocab_rows(const VocabArgs& v, int n_sm, cudaStream_t s);
+// stall, check: bounds of its waits in SM cycles, as in SegPlan.  When one runs
+// out the token is -1, the signals are NaN, and so are the logits of the CTA.
+cudaError_t launch_vocab_rows(const VocabArgs& v, int n_sm, long long stall, long long check, cudaStream_t s);
 cudaError_t launch_kvfill(const DevModel& m, int exit_layer, int grid_x, bool whole, bool pdl, cudaStream_t s);
 // Deferred fill (EE_OPT_LAZY_FILL): an exit step only records its residual
 // and exit layer; before a later step runs layers [j0, j1) every pending

@@ -1608,7 +1608,8 @@ constexpr int vr_rows(int d) {  // rows a stage: as many as fit, in whole turns 
                                                  : kSegChunk / (2 * d);
 }
 template <int KC>
-__global__ void __launch_bounds__(kSegThreads, 1) k_vocab_rows(VocabArgs v, int stages, int rows) {
+__global__ void __launch_bounds__(kSegThreads, 1)
+    k_vocab_rows(VocabArgs v, int stages, int rows, long long stall, long long check) {
     extern __shared__ __align__(128) uint8_t vr_smem[];
     __shared__ int err_local;
     __shared__ float nss[kCW];
@@ -1626,7 +1627,7 @@ __global__ void __launch_bounds__(kSegThreads, 1) k_vocab_rows(VocabArgs v, int 
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    const Waits wt{&err_local, kSegStallCycles, kSegCheckCycles};
+    const Waits wt{&err_local, stall, check};
     const int r0 = (int)((int64_t)v.V * blockIdx.x / gridDim.x), r1 = (int)((int64_t)v.V * (blockIdx.x + 1) / gridDim.x);
     if (threadIdx.x >= kCT) {  // producer
         if (threadIdx.x != kCT) return;
@@ -1710,6 +1711,14 @@ __global__ void __launch_bounds__(kSegThreads, 1) k_vocab_rows(VocabArgs v, int 
         cs.release();
     }
     update();
+    csync();
+    if (*wt.err) {
+        // A wait ran out: rows are missing, and a stage may have been refilled
+        // under a warp that still read it.  None of the CTA's rows count.
+        st.poison();
+        if (v.logits)
+            for (int r = r0 + threadIdx.x; r < r1; r += kCT) v.logits[r] = NAN;
+    }
     vocab_finish(v, st, false, kCW, [] { csync(); });
 }
 
@@ -1744,14 +1753,14 @@ cudaError_t launch_vocab_ring(const VocabArgs& v, const VocabRing& vr, bool pdl,
     return cudaLaunchKernelEx(&cfg, k_vocab_ring, v, vr.stages);
 }
 
-cudaError_t launch_vocab_rows(const VocabArgs& v, int n_sm, cudaStream_t s) {
+cudaError_t launch_vocab_rows(const VocabArgs& v, int n_sm, long long stall, long long check, cudaStream_t s) {
     if (v.d > kVocabRowsMaxD || v.d % 8 || v.mode != 0) return cudaErrorInvalidValue;
     constexpr int stages = 6;
     const size_t smem = stages * (size_t)(kSegChunk + 16);
     auto go = [&](auto kern) -> cudaError_t {
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        kern<<<n_sm, kSegThreads, smem, s>>>(v, stages, vr_rows(v.d));
+        kern<<<n_sm, kSegThreads, smem, s>>>(v, stages, vr_rows(v.d), stall, check);
         return cudaGetLastError();
     };
     if (v.d <= 512) return go(k_vocab_rows<2>);

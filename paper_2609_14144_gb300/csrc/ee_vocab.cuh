@@ -46,6 +46,13 @@ struct SoftStats {
             if (l > m2) m2 = l;
         }
     }
+    // A set that is not known: no token and no number comes out of any merge
+    // with it.
+    __device__ __forceinline__ void poison() {
+        m = INFINITY;
+        s = t = m2 = g = NAN;
+        a = -1;
+    }
     // Merge another set (its indices all differ from this one's).
     __device__ __forceinline__ void merge(const SoftStats& o) {
         if (o.s == 0.f) return;

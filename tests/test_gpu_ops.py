@@ -229,6 +229,44 @@ def test_vocab_signals_tie_and_uniform():
     assert abs(got[0] - 1.0 / V) <= 1e-9 and abs(got[2] + math.log(V)) <= 1e-4
 
 
+@pytest.mark.parametrize("d", [896, 2048])
+def test_vocab_rows_wait_that_runs_out_poisons_the_result(d):
+    """With the bound of its waits lowered to one SM cycle the row-major pass
+    cannot read all of its rows: no token, no signals, no stale logits.  The
+    next call on the same scratch is right again."""
+    import ctypes
+
+    import torch
+
+    from paper_2609_14144_gb300 import _lib, vocab_signals
+
+    V = 40000
+    g = torch.Generator(device="cuda").manual_seed(d)
+    x = torch.randn(d, generator=g, device="cuda")
+    gain = torch.ones(d, device="cuda").to(torch.bfloat16)
+    U = torch.randn(V, d, generator=g, device="cuda").to(torch.bfloat16)
+    ref = U.double() @ (x.double() / torch.sqrt((x.double() ** 2).mean() + 1e-6))
+    scratch = torch.empty(1 << 16, dtype=torch.uint8, device="cuda")
+    token = torch.zeros(1, dtype=torch.int32, device="cuda")
+    sig = torch.zeros(3, device="cuda")
+    logits = torch.full((V,), 1e9, device="cuda")
+    bounded = _lib.load().ee_vocab_signals_bounded
+    p = ctypes.c_void_p
+    bounded.argtypes = [p, p, p, ctypes.c_int, ctypes.c_int, ctypes.c_float, p, ctypes.c_size_t, p, p, p, p,
+                        ctypes.c_longlong]
+    args = (x.data_ptr(), gain.data_ptr(), U.data_ptr(), V, d, 1e-6, scratch.data_ptr(), scratch.numel(),
+            token.data_ptr(), sig.data_ptr(), logits.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    assert bounded(*args, 0) == _lib.EE_EINVAL
+    assert bounded(*args, 1) == 0
+    torch.cuda.synchronize()
+    assert token.item() == -1 and torch.isnan(sig).all()
+    lost = torch.isnan(logits)
+    assert lost.any() and ((logits - ref).abs()[~lost] <= 1e-3 * ref.abs().max()).all()
+    tok, s2 = vocab_signals(x, gain, U, 1e-6, logits=logits, scratch=scratch)
+    assert tok.item() == ref.argmax().item() and torch.isfinite(s2).all()
+    assert ((logits - ref).abs() <= 1e-5 * ref.abs().max()).all()
+
+
 def test_vocab_confidence_ties_lowest_index():
     import torch
 
