@@ -1543,7 +1543,7 @@ int vocab_standalone(const float* x, const uint16_t* gain, const uint16_t* U, in
     EE_CK(cudaMemsetAsync(v.ticket, 0, 4, s));
     // the ring wants 16-byte rows on 16-byte boundaries (the d_model % 8 that
     // ee_vocab_scratch_bytes checks) and the row's columns in registers
-    if (d_model <= kVocabRowsMaxD)
+    if (vocab_rows_pays(vocab, d_model))
         EE_CK(launch_vocab_rows(v, std::min(nsm, kMaxVocabCtas), wait_cycles ? wait_cycles : kSegStallCycles,
                                 wait_cycles ? std::max(1LL, wait_cycles / 4) : kSegCheckCycles, s));
     else

@@ -170,6 +170,14 @@ cudaError_t launch_vocab(const VocabArgs& v, int grid, bool pdl, cudaStream_t s)
 // The pass over a caller's row-major U fed through a shared-memory ring
 // (ee_persist.cu): one CTA per SM; rows of up to kVocabRowsMaxD columns.
 constexpr int kVocabRowsMaxD = 2048;
+// Where it pays: filling the ring and its shared memory cost a short pass more
+// than the streaming kernel's start (us a call, streaming / ring: 4000 rows of
+// 2048 16.6 / 18.3, 12000 24.8 / 24.9, 16000 28.4 / 26.7; 12000 rows of 1536
+// 22.4 / 22.7, 16000 25.1 / 24.9; 8000 of 896 16.1 / 16.4, 12000 17.9 / 16.7;
+// 16000 of 256 15.3 / 15.7, 24000 16.5 / 15.7).
+constexpr bool vocab_rows_pays(int V, int d) {
+    return d <= kVocabRowsMaxD && (d <= 1024 ? V >= 10000 && (int64_t)V * d >= (5 << 20) : V >= 14000);
+}
 // stall, check: bounds of its waits in SM cycles, as in SegPlan.  When one runs
 // out the token is -1, the signals are NaN, and so are the logits of the CTA.
 cudaError_t launch_vocab_rows(const VocabArgs& v, int n_sm, long long stall, long long check, cudaStream_t s);

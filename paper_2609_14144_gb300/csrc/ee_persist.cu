@@ -1593,21 +1593,24 @@ __global__ void __launch_bounds__(kSegThreads, 1) k_vocab_ring(VocabArgs v, int 
 }
 
 // The vocabulary pass over a caller's row-major U [V, d] (standalone ops).
-// CTA b streams its contiguous rows through the ring, kVrRows rows (at most
-// kSegChunk bytes) a stage; a warp takes whole rows of a stage, kVrBatch at a
-// time, lane = 16-byte column chunks lane, lane + 32, ... (one conflict-free
+// CTA b streams its contiguous rows through the ring, vr_rows of them (at most
+// kSegChunk bytes) a stage; a warp takes whole rows of a stage, B at a time,
+// lane = 16-byte column chunks lane, lane + 32, ... (one conflict-free
 // 512-byte load per step), with the normalised input's columns of those chunks
 // kept in registers for the whole pass (KC of them: d <= 256 KC).  A row's
 // sum ends on the lane of its turn, so that the softmax statistics of 32 rows
-// are updated together.  HBM bounds it (2 V d bytes); a streaming launch of
-// one 512-thread CTA per SM with the loads of one row in flight per warp took
-// 113.1 us a call for 151936 x 1536 (4.1 TB/s), the ring 89.4 us (5.2 TB/s).
-constexpr int kVrBatch = 2;  // rows a warp reduces together
-constexpr int vr_rows(int d) {  // rows a stage: as many as fit, in whole turns of the warps
-    return kSegChunk / (2 * d) >= kCW * kVrBatch ? kSegChunk / (2 * d) / (kCW * kVrBatch) * (kCW * kVrBatch)
-                                                 : kSegChunk / (2 * d);
+// are updated together.  Where fewer than two rows a warp fit a stage, the warps
+// take one each and go on in turn from stage to stage: with pairs of rows from
+// warp 0 on, three of eight warps had none at 1536 columns and four at 2048.
+// HBM bounds it (2 V d bytes); a streaming launch of one 512-thread CTA per SM
+// with the loads of one row in flight per warp takes 113.1 us a call for 151936
+// x 1536 (4.1 TB/s), the ring 82.3 us (5.7 TB/s; 89.0 us in pairs), x 2048 143.4
+// us and 101.4 us (6.1 TB/s; 113.0 us in pairs).
+constexpr int vr_batch(int d) { return kSegChunk / (2 * d) >= 2 * kCW ? 2 : 1; }  // rows a warp reduces together
+constexpr int vr_rows(int d) {  // rows a stage: as many as fit, in whole turns of the warps where they take two
+    return vr_batch(d) == 2 ? kSegChunk / (2 * d) / (2 * kCW) * (2 * kCW) : kSegChunk / (2 * d);
 }
-template <int KC>
+template <int KC, int B>
 __global__ void __launch_bounds__(kSegThreads, 1)
     k_vocab_rows(VocabArgs v, int stages, int rows, long long stall, long long check) {
     extern __shared__ __align__(128) uint8_t vr_smem[];
@@ -1676,27 +1679,32 @@ __global__ void __launch_bounds__(kSegThreads, 1)
         const int nr = min(rows, r1 - rb);
         if (cs.ok) {
 #pragma unroll 1
-            for (int r = w * kVrBatch; r < nr; r += kCW * kVrBatch) {
-                float2 acc[kVrBatch][2];
+            for (int r = (w * B - (rb - r0)) & (kCW * B - 1); r < nr; r += kCW * B) {
+                constexpr int NA = 4 / B;  // running sums of a row and lane (pairs)
+                float2 acc[B][NA];
 #pragma unroll
-                for (int b = 0; b < kVrBatch; ++b) acc[b][0] = acc[b][1] = make_float2(0.f, 0.f);
+                for (int b = 0; b < B; ++b)
+#pragma unroll
+                    for (int e = 0; e < NA; ++e) acc[b][e] = make_float2(0.f, 0.f);
 #pragma unroll
                 for (int k = 0; k < KC; ++k) {
                     if (lane + 32 * k < Rc) {
 #pragma unroll
-                        for (int b = 0; b < kVrBatch; ++b) {
-                            // (a row past the stage's rows reads the ring's next bytes: not used)
+                        for (int b = 0; b < B; ++b) {
+                            // (a row past the stage's last: that one again, not used)
                             const uint4 u = lds128(base + min(r + b, nr - 1) * v.d * 2 + k * 512);
-                            acc[b][0] = fma2(make_float2(bflo(u.x), bfhi(u.x)), x[k][0], acc[b][0]);
-                            acc[b][1] = fma2(make_float2(bflo(u.y), bfhi(u.y)), x[k][1], acc[b][1]);
-                            acc[b][0] = fma2(make_float2(bflo(u.z), bfhi(u.z)), x[k][2], acc[b][0]);
-                            acc[b][1] = fma2(make_float2(bflo(u.w), bfhi(u.w)), x[k][3], acc[b][1]);
+                            const uint32_t u4[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                acc[b][e % NA] = fma2(make_float2(bflo(u4[e]), bfhi(u4[e])), x[k][e], acc[b][e % NA]);
                         }
                     }
                 }
 #pragma unroll
-                for (int b = 0; b < kVrBatch; ++b) {
-                    const float t = warp_sum((acc[b][0].x + acc[b][0].y) + (acc[b][1].x + acc[b][1].y));
+                for (int b = 0; b < B; ++b) {
+                    float2 a = add2(acc[b][0], acc[b][1]);
+                    if constexpr (NA == 4) a = add2(a, add2(acc[b][2], acc[b][3]));
+                    const float t = warp_sum(a.x + a.y);
                     if (r + b < nr) {
                         if (lane == turn) {
                             mine = t;
@@ -1705,7 +1713,7 @@ __global__ void __launch_bounds__(kSegThreads, 1)
                         ++turn;
                     }
                 }
-                if (turn > 32 - kVrBatch) update();
+                if (turn > 32 - B) update();
             }
         }
         cs.release();
@@ -1755,6 +1763,7 @@ cudaError_t launch_vocab_ring(const VocabArgs& v, const VocabRing& vr, bool pdl,
 
 cudaError_t launch_vocab_rows(const VocabArgs& v, int n_sm, long long stall, long long check, cudaStream_t s) {
     if (v.d > kVocabRowsMaxD || v.d % 8 || v.mode != 0) return cudaErrorInvalidValue;
+    static_assert(vr_batch(1024) == 2 && vr_batch(1032) == 1, "rows a warp takes at once, below");
     constexpr int stages = 6;
     const size_t smem = stages * (size_t)(kSegChunk + 16);
     auto go = [&](auto kern) -> cudaError_t {
@@ -1763,10 +1772,10 @@ cudaError_t launch_vocab_rows(const VocabArgs& v, int n_sm, long long stall, lon
         kern<<<n_sm, kSegThreads, smem, s>>>(v, stages, vr_rows(v.d), stall, check);
         return cudaGetLastError();
     };
-    if (v.d <= 512) return go(k_vocab_rows<2>);
-    if (v.d <= 1024) return go(k_vocab_rows<4>);
-    if (v.d <= 1536) return go(k_vocab_rows<6>);
-    return go(k_vocab_rows<8>);
+    if (v.d <= 512) return go(k_vocab_rows<2, 2>);
+    if (v.d <= 1024) return go(k_vocab_rows<4, 2>);
+    if (v.d <= 1536) return go(k_vocab_rows<6, 1>);
+    return go(k_vocab_rows<8, 1>);
 }
 
 bool seg_plan(const DevModel& m, int n_sm, SegPlan& p) {

@@ -131,12 +131,13 @@ def test_vocab_confidence(V, d):
         assert int(tok.item()) == c["argmax"]
 
 
-@pytest.mark.parametrize("V", [2, 151, 2433, 20011])
+@pytest.mark.parametrize("V", [2, 151, 2433, 9999, 10001, 13999, 14001, 20011, 20481])
 @pytest.mark.parametrize("d", [256, 264, 512, 520, 1024, 1032, 1536, 1544, 2040, 2048, 2056])
 def test_vocab_rows_widths(V, d):
-    """Row widths at the edges of the columns a lane keeps in registers, ragged
-    last column chunks, fewer rows than CTAs, partly filled stages, and the
-    first width past the ring's.  Logits within the fp32 summation bound, the
+    """Row widths at the edges of the columns a lane keeps in registers and of
+    the rows a warp takes at once, ragged last column chunks, partly filled
+    stages, fewer rows than CTAs, and on both sides of the row counts and
+    widths from which the ring takes over from the streaming kernel.  Logits within the fp32 summation bound, the
     token the highest logit's lowest index."""
     import torch
 
