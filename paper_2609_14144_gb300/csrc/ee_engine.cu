@@ -237,6 +237,7 @@ struct ee_ctx {
     SegPlan seg{};
     bool vring_ok = false;  // ring-fed vocabulary pass supported (used with the persistent layers)
     VocabRing vring{};
+    bool umma_ok = false;   // tcgen05 batches supported
     bool use_rows = false;  // EE_OPT_ROWS: prompt and re-pass in batches of positions
     bool lazy_fill = false; // EE_OPT_LAZY_FILL: skipped layers' entries filled by the next step that runs them
     RowsBuf rows{};
@@ -866,8 +867,9 @@ int ee_create(const ee_model_config* cfg, void* d_workspace, size_t workspace_by
     c->rows.n_sm = c->n_sm;
     c->rows.err = &c->d_ctl->err;
     // prompts and re-passes in batches on the tcgen05 tensor cores where available
-    c->rows.umma = umma_available() ? 1 : 0;
-    c->use_rows = c->rows.umma == 1;
+    c->umma_ok = configure_umma();
+    c->rows.umma = c->umma_ok ? 1 : 0;
+    c->use_rows = c->umma_ok;
 
     const int kmax = std::max({2 * m.d, m.A * m.D, m.F});
     if (configure_kernels(kmax) != cudaSuccess || configure_fill_pending(m.d) != cudaSuccess ||
@@ -1084,7 +1086,7 @@ int ee_set_option(ee_ctx* c, int option, int value) {
             return EE_OK;
         case EE_OPT_ROWS:
             if (value < 0 || value > 2) return fail(EE_EINVAL, "EE_OPT_ROWS takes 0, 1 or 2");
-            if (value == 1 && !umma_available())
+            if (value == 1 && !c->umma_ok)
                 return fail(EE_EINVAL, "the tcgen05 projections are not available on this device");
             c->use_rows = value != 0;
             c->rows.umma = value == 1 ? 1 : 0;

@@ -302,11 +302,12 @@ int64_t rows_part_floats(int d, int A, int KH, int D, int F);
 // after its cache entries, which is all that anything reads of it.
 cudaError_t rows_pass(const DevModel& m, const RowsBuf& b, const int* start, int M, int32_t* d_pos,
                       const int32_t* ids, int pos_base, int t_max, int last_row, cudaStream_t s);
-// tcgen05 projections of the multi-position pass (ee_umma.cu): available on
-// this device (tensor-map encoding and the kernel's shared memory), the K
-// splits for n_sm SMs, and one projection into part[S][M][Np] (the layout of
-// the warp-level path).
-bool umma_available();
+// tcgen05 projections of the multi-position pass (ee_umma.cu): set up on the
+// current device, for each context (false: not available there; the kernels'
+// shared-memory limits, the attention's too, belong to a device), the K splits
+// for n_sm SMs, and one projection into part[S][M][Np] (the layout of the
+// warp-level path).
+bool configure_umma();
 int umma_splits(int64_t n_tiles, int K, int M, int n_sm);
 cudaError_t launch_mm_umma(const uint16_t* W, int64_t n_rows, int K, const uint16_t* x3, int ldx, int M, int S, int n_sm,
                            float* part, int Np, int* err, cudaStream_t s);

@@ -385,26 +385,20 @@ bool small_batch(int M) { return x3_rows(M) <= USmall::rows; }
 
 }  // namespace
 
-bool umma_available() {
-    static int ok = -1;
-    if (ok < 0) {
-        int dev = 0, major = 0, minor = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
-        cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev);
-        CUtensorMap probe;
-        static uint16_t dummy[64 * 8] __attribute__((aligned(16)));
-        ok = major == 10 && encode_fn() && weight_map(&probe, dummy, 4, 64) &&
-             cudaFuncSetAttribute(k_rows_umma<ULarge>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ULarge::smem) ==
-                 cudaSuccess &&
-             cudaFuncSetAttribute(k_rows_umma<UShort>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)UShort::smem) ==
-                 cudaSuccess &&
-             cudaFuncSetAttribute(k_rows_umma<USmall>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)USmall::smem) ==
-                 cudaSuccess &&
-             configure_uattn() == cudaSuccess;
-        cudaGetLastError();
-    }
-    return ok == 1;
+bool configure_umma() {
+    int dev = 0, major = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
+    CUtensorMap probe;
+    static const uint16_t dummy[64 * 8] __attribute__((aligned(16))) = {};
+    auto smem = [](auto kern, size_t bytes) {
+        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+    };
+    const bool ok = major == 10 && encode_fn() && weight_map(&probe, dummy, 4, 64) &&
+                    smem(k_rows_umma<ULarge>, ULarge::smem) && smem(k_rows_umma<UShort>, UShort::smem) &&
+                    smem(k_rows_umma<USmall>, USmall::smem) && configure_uattn() == cudaSuccess;
+    cudaGetLastError();
+    return ok;
 }
 
 // K splits: as many as keep the grid within one wave (one CTA per SM: the
