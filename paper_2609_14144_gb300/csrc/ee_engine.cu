@@ -876,8 +876,8 @@ int ee_create(const ee_model_config* cfg, void* d_workspace, size_t workspace_by
         configure_rows() != cudaSuccess)
         return bail(fail(EE_ECUDA, "kernel configuration failed"));
     c->attn_cluster = attention_cluster_size(m.D, m.KH);
-    if (seg_plan(m, c->n_sm, c->seg) && configure_layers(c->seg.smem) == cudaSuccess &&
-        layers_blocks_per_sm(c->seg.smem) >= 1) {
+    if (seg_plan(m, c->n_sm, c->seg) && configure_layers(c->seg) == cudaSuccess &&
+        layers_blocks_per_sm(c->seg) >= 1) {
         c->seg.dpart = (Tagged*)(w + l.seg_dpart);
         c->seg.opart = (Tagged*)(w + l.seg_opart);
         c->seg.attn_part = (Tagged*)(w + l.seg_attn);

@@ -225,6 +225,9 @@ struct SegPlan {
     int max_splits;         // attention splits per kv head any step can use (at most)
     int rows_per_kv_chunk;  // cache positions per ring chunk
     int max_items;          // O / down-projection items per CTA (at most)
+    bool padded;            // the first layout of shared memory (of three; the kernel has it compiled in)
+    int sc_ld;              // floats of a position's attention scores in shared memory
+    int red_slots;          // tiles whose partial sums wait for one meeting of the warps (at most)
     int n_tiles[4], n_chunks[4], K[4];  // Q/K/V, O, gate/up, down
     // Values handed between CTAs, each a Tagged word (zero after ee_reset):
     Tagged* dpart;          // down-projection partials [tile][n_chunks][32]
@@ -241,8 +244,8 @@ struct SegPlan {
 // Geometry and shared-memory plan for `m` on n_sm SMs (pointers left
 // unset); false if the shape is outside what the kernel supports.
 bool seg_plan(const DevModel& m, int n_sm, SegPlan& p);
-cudaError_t configure_layers(size_t smem);
-int layers_blocks_per_sm(size_t smem);
+cudaError_t configure_layers(const SegPlan& p);
+int layers_blocks_per_sm(const SegPlan& p);
 // Layers [j0, j1) of the step at ctl->pos; `first`: layer j0 takes the
 // embedding of ctl->in_tok.  A cooperative launch of p.G CTAs.
 cudaError_t launch_layers(const DevModel& m, const SegPlan& p, int j0, int j1, int first, cudaStream_t s);

@@ -181,6 +181,7 @@ __device__ __forceinline__ uint32_t lds32(uint32_t a) {
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
     return v;
 }
+__device__ __forceinline__ float lds32f(uint32_t a) { return __uint_as_float(lds32(a)); }
 
 __device__ __forceinline__ void sts64(uint32_t a, uint32_t x, uint32_t y) {
     asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(a), "r"(x), "r"(y) : "memory");
@@ -405,15 +406,16 @@ struct Smem {
     float* xa;          // [max items][512] staged input columns of the O / down items, then
                         // [max items][32] residual rows of the O items of chunk 0
     float2* rope;       // [D/2] (cos, sin) of the step's position
-    float* red;         // [kRedSlots][kCW][32], then [kCW] sums of squares of the RMSNorm
-    float* qa;          // [group][D] scaled queries of the attention unit
+    float* red;         // [red_slots][kCW][32]
+    float* nss;         // [kCW] sums of squares of the RMSNorm
     float* kv;          // [2][D] k, v of the step's position
-    float* sc;          // [pps * page_size][sc_heads(group)] scores, then probabilities
+    float* sc;          // [pps * page_size][sc_ld] scores, then probabilities
     float* ml;          // [group][2] max, sum
     uint8_t* nsd;       // [down tiles] slots per down tile
 };
 // Heads of a score row: the group rounded up to 4, so that a position's
-// probabilities of four heads are one 16-byte load.
+// probabilities of four heads are one 16-byte load (PAD); the group itself where
+// that row is too long for the context (seg_plan).
 __host__ __device__ constexpr int sc_heads(int grp) { return (grp + 3) & ~3; }
 __device__ __forceinline__ Smem carve(uint8_t* base, const DevModel& m, const SegPlan& p) {
     Smem s;
@@ -432,16 +434,15 @@ __device__ __forceinline__ Smem carve(uint8_t* base, const DevModel& m, const Se
     s.rope = reinterpret_cast<float2*>(f);
     f += m.D;
     s.red = f;
-    f += kRedSlots * kCW * 32 + kCW;
-    const int grp = m.A / m.KH;
-    s.qa = f;
-    f += grp * m.D;
+    f += p.red_slots * kCW * 32;
+    s.nss = f;
+    f += kCW;
     s.kv = f;
     f += 2 * m.D;
     s.sc = f;
-    f += sc_heads(grp) * p.max_pps * m.page_size;
+    f += p.sc_ld * p.max_pps * m.page_size;
     s.ml = f;
-    f += 2 * grp;
+    f += 2 * (m.A / m.KH);
     s.nsd = reinterpret_cast<uint8_t*>(f);
     return s;
 }
@@ -725,16 +726,16 @@ __device__ __forceinline__ float gather_norm(float* xs, const uint16_t* g, int d
 // Whole tiles [t0, t1) of a matrix with rows of length K against x (all K
 // columns in shared memory).  epi(t, s) runs in one warp with lane = row of
 // the tile and s its complete dot product.  The warps' partial sums of up to
-// kRedSlots tiles meet at one barrier and the epilogues run in different
+// `slots` (at most kCW) tiles meet at one barrier and the epilogues run in different
 // warps: with a barrier and an epilogue in warp 0 for every tile, warp 0 held
 // up the other seven.  (Callers have a consumer barrier between one call's
 // epilogues and the next call.)
 template <class Epi>
-__device__ __forceinline__ void tile_gemv(Consumer& cs, int t0, int t1, int K, int nc, const float* x, float* red, Epi epi) {
+__device__ __forceinline__ void tile_gemv(Consumer& cs, int t0, int t1, int K, int nc, const float* x, float* red, int slots, Epi epi) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll 1
-    for (int tb = t0; tb < t1; tb += kRedSlots) {
-        const int te = min(t1, tb + kRedSlots);
+    for (int tb = t0; tb < t1; tb += slots) {
+        const int te = min(t1, tb + slots);
 #pragma unroll 1
         for (int t = tb; t < te; ++t) {
             RowAcc acc;
@@ -815,12 +816,12 @@ __device__ __forceinline__ float4 resid_mid4(const SegPlan& p, const Tagged* opa
 // The attention unit of one CTA: kv head g, cached positions [p0, p1) of
 // [0, pos], for the group's query heads; writes the split's unnormalised
 // output, maximum and sum per head.
-template <int D>
+template <int D, bool PAD>
 __device__ __forceinline__ void attn_phase(const DevModel& m, const SegPlan& p, const Smem& s, Consumer& cs, Poll& pl,
                                            const AttnGeo& ag, int unit, int pos, uint32_t tag) {
     constexpr int kPairs = D / 32;  // pairs of k16 steps (32 dimensions)
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int grp = m.A / m.KH, gp = sc_heads(grp);
+    const int grp = m.A / m.KH, gp = PAD ? sc_heads(grp) : p.sc_ld;
     const int rpc = p.rows_per_kv_chunk;
     const int g = unit / ag.splits, sp = unit - g * ag.splits;
     const int p0 = sp * ag.pps * m.page_size, p1 = min(ag.T, min(ag.n_pages, (sp + 1) * ag.pps) * m.page_size);
@@ -957,12 +958,13 @@ __device__ __forceinline__ void attn_phase(const DevModel& m, const SegPlan& p, 
     // P V: warp w takes the four heads from 4 hg on, hg = w / npq, and the
     // positions r = w mod npq (mod npq); lane = dpl dimensions.  Each V row is
     // read once per four heads, with one load for its four probabilities (those
-    // past the group are garbage, multiplied into sums nobody reads).  The npq
+    // past the group are garbage, multiplied into sums nobody reads; four loads
+    // where the rows are not padded).  The npq
     // partial sums per head meet in shared memory (xs and xa, contiguous and
     // free here) and are added in order.
     constexpr int dpl = D / 32;  // 2 or 4
     const int avail = ((max(m.d, m.A * D) + 3) & ~3) + p.max_items * (kColsPerChunk + 32);
-    int npq = kCW / (gp >> 2);
+    int npq = kCW / (sc_heads(grp) >> 2);
 #pragma unroll 1
     while (npq > 1 && npq * grp * D > avail) npq >>= 1;
     const int hg = w / npq, pq = w - hg * npq;
@@ -987,9 +989,13 @@ __device__ __forceinline__ void attn_phase(const DevModel& m, const SegPlan& p, 
                 __syncwarp();
             }
             const uint32_t va = vst + lane * dpl * 2, pa = saddr(s.sc + (base - p0) * gp + hg * 4);
+            const int past = 4 * (gp - 1 - 4 * hg);  // byte offset of the row's last head (not padded)
 #pragma unroll 4
             for (int r = pq; r < nr; r += npq) {
-                const float4 pr = lds128f(pa + r * gp * 4);
+                const uint32_t pr_at = pa + r * gp * 4;
+                const float4 pr = PAD ? lds128f(pr_at)
+                                      : make_float4(lds32f(pr_at), lds32f(pr_at + min(4, past)),
+                                                    lds32f(pr_at + min(8, past)), lds32f(pr_at + min(12, past)));
                 float v[dpl];
                 if (dpl == 4) {
                     const uint2 u = lds64(va + r * D * 2);
@@ -1043,6 +1049,7 @@ __device__ __forceinline__ void attn_phase(const DevModel& m, const SegPlan& p, 
 
 }  // namespace
 
+template <bool PAD>
 __global__ void __launch_bounds__(kSegThreads, 1) k_layers(DevModel m, SegPlan p, int j0, int j1, int first) {
     extern __shared__ __align__(128) uint8_t seg_smem[];
     const Smem s = carve(seg_smem, m, p);
@@ -1209,12 +1216,12 @@ __global__ void __launch_bounds__(kSegThreads, 1) k_layers(DevModel m, SegPlan p
                 pl.probe(p.dpart + (last_dn_slot + s.nsd[p.n_tiles[3] - 1] - 1) * 32 + 31, seq_tag(seq - 1));
             else
                 csync();
-            const float inv = gather_norm<2>(s.xs, lw + m.off_gattn, m.d, m.eps, s.red + kRedSlots * kCW * 32, pl,
+            const float inv = gather_norm<2>(s.xs, lw + m.off_gattn, m.d, m.eps, s.nss, pl,
                                           [&](int i, uint32_t& bad) { return rin.four(i, bad); });
             const uint16_t* bias = m.qkv_bias ? lw + m.off_bqkv : nullptr;
             uint16_t* kdst = m.kpool + (int64_t)j * m.kv_layer_stride + kvo_pos;
             uint16_t* vdst = m.vpool + (int64_t)j * m.kv_layer_stride + kvo_pos;
-            tile_gemv(cs, tq0, tq1, p.K[0], p.n_chunks[0], s.xs, s.red, [&](int t, float v) {
+            tile_gemv(cs, tq0, tq1, p.K[0], p.n_chunks[0], s.xs, s.red, PAD ? kRedSlots : p.red_slots, [&](int t, float v) {
                 const int odd = lane & 1;
                 const int u = t * 16 + (lane >> 1);
                 v *= inv;
@@ -1253,9 +1260,9 @@ __global__ void __launch_bounds__(kSegThreads, 1) k_layers(DevModel m, SegPlan p
         // ---------------- attention unit (if this CTA has one)
         if (unit >= 0) {
             if (m.D == 128)
-                attn_phase<128>(m, p, s, cs, pl, ag, unit, pos, tag);
+                attn_phase<128, PAD>(m, p, s, cs, pl, ag, unit, pos, tag);
             else
-                attn_phase<64>(m, p, s, cs, pl, ag, unit, pos, tag);
+                attn_phase<64, PAD>(m, p, s, cs, pl, ag, unit, pos, tag);
         }
 
         // ---------------- O items: merge the attention splits of the chunk's heads,
@@ -1407,9 +1414,9 @@ __global__ void __launch_bounds__(kSegThreads, 1) k_layers(DevModel m, SegPlan p
         // ---------------- gate/up tiles: RMSNorm of the mid residual, SwiGLU
         if (tg1 > tg0) {
             pl.probe(op_cur + ((int64_t)p.n_tiles[1] * p.n_chunks[1] - 1) * 32 + 31, tag);  // the last O slot
-            const float inv = gather_norm<2>(s.xs, lw + m.off_gmlp, m.d, m.eps, s.red + kRedSlots * kCW * 32, pl,
+            const float inv = gather_norm<2>(s.xs, lw + m.off_gmlp, m.d, m.eps, s.nss, pl,
                                           [&](int i, uint32_t& bad) { return resid_mid4(p, op_cur, i, tag, bad); });
-            tile_gemv(cs, tg0, tg1, p.K[2], p.n_chunks[2], s.xs, s.red, [&](int t, float v) {
+            tile_gemv(cs, tg0, tg1, p.K[2], p.n_chunks[2], s.xs, s.red, PAD ? kRedSlots : p.red_slots, [&](int t, float v) {
                 v *= inv;
                 const float up = __shfl_xor_sync(0xffffffffu, v, 1);
                 const int f = t * 16 + (lane >> 1);
@@ -1582,7 +1589,7 @@ __global__ void __launch_bounds__(kSegThreads, 1) k_vocab_ring(VocabArgs v, int 
     }
     const bool keep = v.logits && (!v.logits_if_dbg || (v.ctl && v.ctl->dbg));
     SoftStats st;  // warp w keeps the statistics of the tiles whose rows it finishes
-    tile_gemv(cs, t0, t1, v.d, nc, xs, red, [&](int t, float sum) {
+    tile_gemv(cs, t0, t1, v.d, nc, xs, red, kRedSlots, [&](int t, float sum) {
         const int row = t * kTileRows + lane;
         if (row < v.V) {
             if (keep) v.logits[row] = sum;
@@ -1807,13 +1814,25 @@ bool seg_plan(const DevModel& m, int n_sm, SegPlan& p) {
     const int np_max = (m.max_ctx + m.page_size - 1) / m.page_size;
     p.max_pps = std::max(1, (np_max + cap - 1) / cap);
     p.max_splits = std::min(cap, np_max);
-    // xs, xa, rope, red (+ norm partials), qa, kv, sc, ml (the carve above)
-    const size_t floats = (size_t)((std::max(m.d, m.A * m.D) + 3) & ~3) + (size_t)p.max_items * (kColsPerChunk + 32) +
-                          (size_t)m.D + kRedSlots * kCW * 32 + kCW + (size_t)grp * m.D + 2 * (size_t)m.D +
-                          (size_t)sc_heads(grp) * p.max_pps * m.page_size + 2 * (size_t)grp;
-    const size_t fixed = floats * 4 + (size_t)p.n_tiles[3] + 256;
+    // xs, xa, rope, red, norm partials, kv, sc, ml (the carve above).  Padded score
+    // rows and all partial-sum slots if they fit, else rows of the group's
+    // heads, else half the slots too: the longest context that the kernel takes is
+    // the last layout's (1.5B, pages of 64: 151552, 200704 and 204800 positions).
+    const int layouts[3][2] = {{sc_heads(grp), kRedSlots}, {grp, kRedSlots}, {grp, kRedSlots / 2}};
     const size_t budget = 227 * 1024;
-    if (fixed + 4 * (size_t)(kSegChunk + 16) > budget) return false;
+    size_t floats = 0, fixed = 0;
+    bool fits = false;
+    for (int i = 0; i < 3 && !fits; ++i) {
+        p.sc_ld = layouts[i][0];
+        p.red_slots = layouts[i][1];
+        p.padded = i == 0;
+        floats = (size_t)((std::max(m.d, m.A * m.D) + 3) & ~3) + (size_t)p.max_items * (kColsPerChunk + 32) + (size_t)m.D +
+                 (size_t)p.red_slots * kCW * 32 + kCW + 2 * (size_t)m.D + (size_t)p.sc_ld * p.max_pps * m.page_size +
+                 2 * (size_t)grp;
+        fixed = floats * 4 + (size_t)p.n_tiles[3] + 256;
+        fits = fixed + 4 * (size_t)(kSegChunk + 16) <= budget;
+    }
+    if (!fits) return false;
     // the attention unit's three bf16 parts of the group's queries fit in xs
     if ((size_t)3 * grp * (m.D + 8) * 2 > (size_t)4 * ((std::max(m.d, m.A * m.D) + 3) & ~3)) return false;
     p.stages = (int)std::min<size_t>(16, (budget - fixed) / (kSegChunk + 16));
@@ -1822,13 +1841,16 @@ bool seg_plan(const DevModel& m, int n_sm, SegPlan& p) {
     return true;
 }
 
-cudaError_t configure_layers(size_t smem) {
-    return cudaFuncSetAttribute(k_layers, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+cudaError_t configure_layers(const SegPlan& p) {
+    return cudaFuncSetAttribute(p.padded ? k_layers<true> : k_layers<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)p.smem);
 }
 
-int layers_blocks_per_sm(size_t smem) {
+int layers_blocks_per_sm(const SegPlan& p) {
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_layers, kSegThreads, smem) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, p.padded ? k_layers<true> : k_layers<false>, kSegThreads, p.smem) !=
+        cudaSuccess)
+        return 0;
     return n;
 }
 
@@ -1843,7 +1865,7 @@ cudaError_t launch_layers(const DevModel& m, const SegPlan& p, int j0, int j1, i
     at[0].val.cooperative = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_layers, m, p, j0, j1, first);
+    return cudaLaunchKernelEx(&cfg, p.padded ? k_layers<true> : k_layers<false>, m, p, j0, j1, first);
 }
 
 }  // namespace ee

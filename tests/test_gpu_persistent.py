@@ -7,7 +7,7 @@ import pytest
 
 import oracle
 import synth
-from helpers import check_kv, check_records, gpu_replay, oracle_steps, teacher_forced
+from helpers import check_kv, check_records, gpu_replay, oracle_steps, rel_err, teacher_forced
 
 pytestmark = pytest.mark.gpu
 
@@ -101,6 +101,36 @@ def test_1p5b_persistent_agrees_with_five_launch_path():
     first_diff = np.argmax(~agree) if not agree.all() else len(agree)
     assert first_diff == len(agree) or near[first_diff]
     assert np.max(np.abs(c0[:first_diff] - c1[:first_diff]), initial=0) < 1e-3
+
+
+@pytest.mark.parametrize("G,max_ctx", [(1, 200000), (1, 440000), (2, 150000), (3, 100000), (5, 60000), (5, 80000),
+                                       (6, 60000), (6, 65000), (7, 50000), (7, 54000)])
+def test_long_contexts_keep_the_persistent_layers(G, max_ctx):
+    """Contexts whose attention scores fit beside the ring only in rows of the
+    group's own heads (groups that are not a multiple of 4), or with half the
+    partial-sum slots besides (the second length of a group): eight key-value
+    heads of 64, several pages to a split.  The layers stay persistent and agree
+    with the five-launch path."""
+    from paper_2609_14144_gb300 import OPT_DEBUG_LOGITS, OPT_PERSISTENT, Engine
+
+    shape = TINY.replace(n_heads=8 * G, n_kv_heads=8, n_layers=2, readout_layers=(1,))
+    model = synth.make_model(shape)
+    prompt = synth.token_ids(shape.seed, 940, 1500, shape.vocab)
+    got = []
+    for pers in (1, 0):
+        eng = Engine(shape, model, max_ctx=max_ctx)
+        assert eng.persistent
+        eng.set_option(OPT_PERSISTENT, pers)
+        eng.set_option(OPT_DEBUG_LOGITS, 1)
+        eng.prefill(prompt)
+        out = []
+        for tok in (5, 6, 7):
+            eng.decode_step(tok, [2.0], oracle.FORCE_FULL)
+            out.append((eng.hidden_final(), eng.final_logits()))
+        got.append(out)
+        eng.close()
+    for a, b in zip(*got):
+        assert rel_err(a[0], b[0]) <= 1e-3 and rel_err(a[1], b[1]) <= 1e-3
 
 
 def test_ring_products_round_like_short_chains():
