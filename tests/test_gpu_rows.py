@@ -1,7 +1,7 @@
 """The multi-position layer pass on the GPU (needs a GB300).
 
 With EE_OPT_ROWS = 1 the prompt and the re-pass run each layer over batches
-of up to 256 positions, the projections on the tcgen05 tensor cores (2: the
+of up to ROWS_MAX positions, the projections on the tcgen05 tensor cores (2: the
 same batches with warp-level mma products).  Checked against the oracle (first token exact outside
 the 1e-3 top-2 band, final hidden state and logits and every cache entry
 within 1e-2 relative, which (layer, position) entries were computed bit for
@@ -9,6 +9,10 @@ bit) and against the same engine one position at a time (EE_OPT_ROWS = 0,
 the default): both keep activations at fp32 precision (the batched products
 through three bf16 parts of each activation), so fp32 results agree within
 1e-3 relative; cache entries are bf16, where one rounding step is 4e-3."""
+import math
+import os
+import re
+
 import numpy as np
 import pytest
 
@@ -19,6 +23,9 @@ from helpers import EXCLUDE_EPS, REL_TOL, bf16_bits_to_f32, check_kv, rel_err, t
 pytestmark = pytest.mark.gpu
 
 TINY = synth.CONFIGS["tiny"]
+_HEADER = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_14144_gb300", "csrc",
+                       "ee_internal.h")
+ROWS_MAX = int(re.search(r"kRowsMax = (\d+);", open(_HEADER).read()).group(1))  # positions per batch
 PATH_TOL = 1e-3  # fp32 results of the batched and the one-position paths
 
 
@@ -47,13 +54,14 @@ def _engine(shape, model, max_ctx, rows=True, pages=None):
 
 
 @pytest.mark.parametrize("mode", [1, 2])
-@pytest.mark.parametrize("n", [1, 7, 16, 17, 255, 256, 257, 600])
+@pytest.mark.parametrize("n", [1, 7, 16, 17, 255, 256, 257, 600, ROWS_MAX - 1, ROWS_MAX, ROWS_MAX + 1, 2 * ROWS_MAX + 88])
 def test_tiny_prompt_batches_match_oracle(tiny_model, n, mode):
     """Prompts of one position, a partial first group of 16 rows (the
     tcgen05 products' N step), one full group, a full group and one row, one
-    short of a full batch, one full batch, a full batch and one position, and
-    two full batches and a ragged tail, on the tcgen05 and the warp-level
-    products (F = 688: a ragged last K stage)."""
+    short of a full row block (256), one full block, two blocks, three; and one
+    short of a full batch, one full batch, two batches, and three with a ragged
+    tail, on the tcgen05 and the warp-level products (F = 688: a ragged last K
+    stage)."""
     prompt = synth.token_ids(TINY.seed, 901, n, TINY.vocab)
     orc = oracle.Oracle(TINY, tiny_model, max_ctx=n + 1)
     tok_o, cap = orc.prefill(prompt, capture=True)
@@ -108,6 +116,68 @@ def test_tiny_prompt_paths_agree(tiny_model):
             assert ra["token"] == rb["token"]
         assert abs(ra["confidence"][0] - rb["confidence"][0]) <= 5e-4
         tok = rb["token"]
+
+
+def _cut(x, parts):
+    """x as the sum of its first bf16 parts (each the rounding of what is left)."""
+    out, rest = np.zeros_like(x), x.astype(np.float32)
+    for _ in range(parts):
+        p = bf16_bits_to_f32(to_bf16_bits(rest))
+        out, rest = out + p, rest - p
+    return out
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("n", [70, 129, 700, 1300])
+@pytest.mark.parametrize("spread,tol", [(1, 6e-7), (150, 3e-6)])
+def test_tcgen05_attention_parts_and_growing_scores(n, D, spread, tol):
+    """The last row's attention of the first layer (16 heads, up to 21 blocks of
+    64 keys) against 64 bits over the engine's own cache.  spread 1: flat
+    probabilities; the third bf16 part of each is 2^-18 of it, 2.2e-6 of the
+    output in the mean.  spread 150: scores tens apart, so that the largest so
+    far comes in early, middle and late blocks, rows of a tile grow their
+    references in different blocks and within chains; the third part of the
+    queries moves a score by 1e-4.  What the fp32 sums, the products of Q and O
+    and the exponentials leave is 4e-7 and 1.5e-6; a reference whose queries or
+    probabilities lack their third part misses the result by more than the
+    bound."""
+    shape = TINY.replace(n_heads=16, head_dim=D, n_layers=2, readout_layers=(1,))
+    model = synth.make_model(shape)
+    for lw in model["layers"]:
+        lw["wd"] = np.zeros_like(lw["wd"])
+    lw = model["layers"][0]
+    lw["wo"] = to_bf16_bits(bf16_bits_to_f32(lw["wo"]) * 50)  # large beside the residual
+    lw["wq"] = to_bf16_bits(bf16_bits_to_f32(lw["wq"]) * spread)
+    model["layers"][1]["wo"] = np.zeros_like(lw["wo"])
+    prompt = synth.token_ids(shape.seed, 960 + n, n, shape.vocab)
+    eng = _engine(shape, model, n + 1)
+    eng.prefill(prompt)
+    A, K = shape.n_heads, shape.n_kv_heads
+    kv = [eng.kv(0, t) for t in range(n)]
+    k, v = (np.stack(x).astype(np.float64).reshape(n, K, D).repeat(A // K, axis=1) for x in zip(*kv))
+    w = {name: synth.bf16_to_f32(lw[name]).astype(np.float64) for name in ("wq", "wo", "attn_norm")}
+    x = synth.bf16_to_f32(model["embed"])[prompt[-1]].astype(np.float64)
+    z = x / np.sqrt((x * x).mean() + np.float32(shape.rms_eps)) * w["attn_norm"]
+    ang = (n - 1) * shape.rope_base ** (-2.0 * np.arange(D // 2) / D)
+    c, s = (f(ang).astype(np.float32).astype(np.float64) for f in (np.cos, np.sin))
+    a, b = (w["wq"] @ z).reshape(A, 2, D // 2).transpose(1, 0, 2)
+    q = np.concatenate([a * c - b * s, a * s + b * c], 1) / math.sqrt(D)
+
+    def attend(q, parts=None):
+        sc = np.einsum("hd,thd->ht", q, k)
+        p = np.exp(sc - sc.max(1, keepdims=True))
+        o = np.einsum("ht,thd->hd", _cut(p, parts) if parts else p, v) / p.sum(1, keepdims=True)
+        return w["wo"] @ o.reshape(-1), sc
+
+    ref, sc = attend(q)
+    off = lambda y: np.linalg.norm(y - ref) / np.linalg.norm(ref)
+    if spread == 1:
+        assert off(attend(q, 2)[0]) > tol
+    else:
+        assert off(attend(_cut(q, 2))[0]) > tol
+        grows = [(h, t) for h in range(A) for t in range(64, n) if sc[h, t] > sc[h, :t // 64 * 64].max() + 8]
+        assert grows or n < 700
+    assert off(eng.hidden_final() - x) <= tol, off(eng.hidden_final() - x)
 
 
 @pytest.mark.parametrize("D,page", [(64, 16), (64, 256), (128, 64), (128, 32)])
@@ -185,23 +255,36 @@ def _exit_decode(shape, model, n, force_of, rows=True):
     return orc, eng
 
 
-def test_tiny_repass_in_several_batches(tiny_model):
-    """450 decoded positions, two of three exited: 300 rows, a full batch and
-    a partial one."""
-    n, P = 450, TINY.prompt_len
-    force = lambda i: oracle.FORCE_FULL if i % 3 == 0 else oracle.FORCE_EXIT_AT(0)
-    orc, eng = _exit_decode(TINY, tiny_model, n, force)
-    assert eng.repass(P, P + n) == orc.repass(P, P + n) == n - (n + 2) // 3
-    check_kv(orc, eng, TINY, P + n)
+@pytest.mark.parametrize("mode", [1, 2])
+def test_tiny_repass_in_several_batches(mode):
+    """More exited positions than a batch holds (two of three of 1.6 ROWS_MAX:
+    a full batch and a partial one), left at three layers in turn: a later batch
+    reads an earlier one's entries, and the last position, which left first, is
+    not the last of its batch's rows."""
+    shape = TINY.replace(readout_layers=(1, 2, 3))
+    model = synth.make_model(shape)
+    n, P = int(1.6 * ROWS_MAX) // 6 * 6 + 2, shape.prompt_len
+    force = lambda i: oracle.FORCE_FULL if i % 3 == 0 else oracle.FORCE_EXIT_AT((n - 1 - i) % 5 % 3)
+    assert force(n - 1) == oracle.FORCE_EXIT_AT(0)
+    orc, eng = _exit_decode(shape, model, n, force, rows=mode)
+    todo = n - (n + 2) // 3
+    assert ROWS_MAX < todo < 2 * ROWS_MAX
+    assert eng.repass(P, P + n) == orc.repass(P, P + n) == todo
+    check_kv(orc, eng, shape, P + n)
+    _, one = _exit_decode(shape, model, n, force, rows=0)
+    assert one.repass(P, P + n) == todo
+    assert rel_err(eng.hidden_final(), one.hidden_final()) <= PATH_TOL  # the last re-passed position's
     assert eng.repass(P, P + n) == 0
 
 
-def test_tiny_repass_rows_starting_at_different_layers():
+@pytest.mark.parametrize("n", [40, 200])
+def test_tiny_repass_rows_starting_at_different_layers(n):
     """Three readouts: exits at layers 1, 2 and 3 in one batch, so rows join
-    the batch at different layers."""
+    the batch at different layers, their positions in no order (200: up to 146
+    rows, on the tcgen05 attention from the second layer on)."""
     shape = TINY.replace(readout_layers=(1, 2, 3))
     model = synth.make_model(shape)
-    n, P = 40, shape.prompt_len
+    P = shape.prompt_len
     force = lambda i: oracle.FORCE_FULL if i % 4 == 3 else oracle.FORCE_EXIT_AT(i % 4)
     orc, eng = _exit_decode(shape, model, n, force)
     assert eng.repass(P + 5, P + n) == orc.repass(P + 5, P + n)
@@ -224,8 +307,8 @@ def test_tiny_repass_paths_agree(tiny_model):
 
 
 def test_1p5b_prompt_batches_sampled():
-    """The 1.5B shape with a 300-position prompt (a full batch and a partial
-    one): first token, final state and sampled cache entries."""
+    """The 1.5B shape with a 300-position prompt (two row blocks): first token,
+    final state and sampled cache entries."""
     shape = synth.CONFIGS["1.5b"].replace(prompt_len=300)
     model = synth.make_model(shape)
     n = 300
@@ -248,8 +331,7 @@ def test_1p5b_prompt_batches_sampled():
 @pytest.mark.parametrize("name", ["0.5b", "1.5b"])
 def test_tensor_core_paths_agree(name):
     """The tcgen05 products (EE_OPT_ROWS = 1) against the warp-level ones
-    (2) on a 256-position batch and a 44-position one: same first token,
-    fp32 states within 1e-3, cache entries within 1e-2 (bf16 rounding)."""
+    (2) on a 300-position batch (two row blocks): same first token, fp32 states within 1e-3, cache entries within 1e-2 (bf16 rounding)."""
     shape = synth.CONFIGS[name].replace(prompt_len=300)
     model = synth.make_model(shape)
     prompt = synth.prompt(shape)
