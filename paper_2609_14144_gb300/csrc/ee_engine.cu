@@ -1475,6 +1475,8 @@ int ee_profile_kernels(ee_ctx* c, int iters, float* ms_out) {
 
 int ee_attention_scratch_bytes(int n_heads, int n_kv_heads, int head_dim, size_t* bytes) {
     if (!bytes || n_heads <= 0 || n_kv_heads <= 0 || (head_dim != 64 && head_dim != 128)) return fail(EE_EINVAL, "bad shape");
+    // (the second part was the arrival counters of an earlier kernel; the sizes
+    // that callers have stored, and what is refused, stay as they were)
     *bytes = align_up(4 * (size_t)n_heads * kAttnMaxSplits * (head_dim + 2)) + align_up(4 * (size_t)n_kv_heads);
     return EE_OK;
 }

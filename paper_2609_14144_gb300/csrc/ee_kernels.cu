@@ -985,10 +985,11 @@ __global__ void __launch_bounds__(kGemvThreads, 2) k_vocab_rowmajor(VocabArgs v)
 // query is read once for both.  P V: lane = D / 32 dimensions, a position's
 // probabilities of all heads are one or two 16-byte loads.  k_attn_merge
 // combines the splits, one CTA per (head, 32 dimensions).
-// A call at 12/2 heads of 128 and 16411 positions takes 18.4 us (of which the
-// host's two launches 18), 96.6 us for a per-lane online softmax over every
-// position with the merge in the last CTA of a head (two exponentials per
-// position and head, and a serial merge of 128 splits).
+// A call at 12/2 heads of 128 and 16411 positions takes 18.6 us on the device,
+// 96.5 us for a per-lane online softmax over every position with the merge in the
+// last CTA of a head (two exponentials per position and head, and a serial merge
+// of 128 splits).  Up to about 6000 positions it takes the two launches' 10 to 12
+// us (14 to 87); the host issues a call in 5.2 us.
 constexpr int kAttnTile = 16;  // positions per warp and tile
 template <int D, int G>
 __global__ void __launch_bounds__(kAttnThreads, 2) k_attn_split(AttnArgs a, int chunk) {

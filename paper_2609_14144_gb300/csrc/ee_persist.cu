@@ -44,6 +44,7 @@
 #include <algorithm>
 
 #include "ee_internal.h"
+#include "ee_split3.cuh"
 #include "ee_vocab.cuh"
 
 namespace ee {
@@ -189,17 +190,6 @@ __device__ __forceinline__ void sts64(uint32_t a, uint32_t x, uint32_t y) {
 // Two floats as bf16 (round to nearest even), the first in the low half.
 __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
     return (uint32_t)tobf(a) | ((uint32_t)tobf(b) << 16);
-}
-// x0, x1 as three packed bf16 parts: high = bf16(x), middle = bf16(x -
-// high), low = bf16(x - high - middle).  Both differences are exact in fp32
-// and the low part holds what is left, so high + middle + low = x.
-__device__ __forceinline__ void split3_bf16x2(float x0, float x1, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
-    const uint16_t h0 = tobf(x0), h1 = tobf(x1);
-    const float r0 = x0 - bf(h0), r1 = x1 - bf(h1);
-    const uint16_t m0 = tobf(r0), m1 = tobf(r1);
-    hi = (uint32_t)h0 | ((uint32_t)h1 << 16);
-    mid = (uint32_t)m0 | ((uint32_t)m1 << 16);
-    lo = pack_bf16x2(r0 - bf(m0), r1 - bf(m1));
 }
 // d += A B for one m16n8k16 tile: bf16 A (4 registers, row-major
 // fragment), bf16 B (2 registers, column-major fragment), fp32 accumulators.
@@ -858,12 +848,11 @@ __device__ __forceinline__ void attn_phase(const DevModel& m, const SegPlan& p, 
             *reinterpret_cast<float4*>(s.kv + (b - nqa)) = v;
         } else {
             const int h = b / D, c = b - h * D;
-            uint32_t h01, m01, l01, h23, m23, l23;
-            split3_bf16x2(v.x * scale, v.y * scale, h01, m01, l01);
-            split3_bf16x2(v.z * scale, v.w * scale, h23, m23, l23);
-            sts64(saddr(qhs + h * qrow + c), h01, h23);
-            sts64(saddr(qhs + (grp + h) * qrow + c), m01, m23);
-            sts64(saddr(qhs + (2 * grp + h) * qrow + c), l01, l23);
+            uint32_t p01[3], p23[3];
+            split3(v.x * scale, v.y * scale, p01);
+            split3(v.z * scale, v.w * scale, p23);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) sts64(saddr(qhs + (k * grp + h) * qrow + c), p01[k], p23[k]);
         }
     }
     csync();

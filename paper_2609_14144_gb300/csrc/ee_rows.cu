@@ -44,6 +44,7 @@
 #include <algorithm>
 
 #include "ee_internal.h"
+#include "ee_split3.cuh"
 
 namespace ee {
 namespace {
@@ -71,32 +72,21 @@ struct Parts {
     }
 };
 
-// Two values as three packed bf16 parts: high = bf16(x), middle = bf16(x -
-// high), low = bf16(x - high - middle) (each difference exact in fp32); four
-// columns of a row stored from `at` on (its high part), and eight (a whole
-// chunk), one store per part.
-__device__ __forceinline__ void split_pair(float a, float b, uint32_t (&p)[3]) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);  // a in the low half
-        p[k] = *reinterpret_cast<const uint32_t*>(&v);
-        a -= __uint_as_float(p[k] << 16);
-        b -= __uint_as_float(p[k] & 0xffff0000u);
-    }
-}
+// Four columns of a row stored as parts from `at` on (its high part), and eight
+// (a whole chunk), one store per part.
 __device__ __forceinline__ void split_store4(float4 x, const Parts& p, int64_t at) {
     uint32_t a[3], b[3];
-    split_pair(x.x, x.y, a);
-    split_pair(x.z, x.w, b);
+    split3(x.x, x.y, a);
+    split3(x.z, x.w, b);
 #pragma unroll
     for (int k = 0; k < 3; ++k) *reinterpret_cast<uint2*>(p.p + at + k * p.rows * 8) = make_uint2(a[k], b[k]);
 }
 __device__ __forceinline__ void split_store8(const float (&x)[8], const Parts& p, int64_t at) {
     uint32_t a[3], b[3], c[3], d[3];
-    split_pair(x[0], x[1], a);
-    split_pair(x[2], x[3], b);
-    split_pair(x[4], x[5], c);
-    split_pair(x[6], x[7], d);
+    split3(x[0], x[1], a);
+    split3(x[2], x[3], b);
+    split3(x[4], x[5], c);
+    split3(x[6], x[7], d);
 #pragma unroll
     for (int k = 0; k < 3; ++k)
         *reinterpret_cast<uint4*>(p.p + at + k * p.rows * 8) = make_uint4(a[k], b[k], c[k], d[k]);

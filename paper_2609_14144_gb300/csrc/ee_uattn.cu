@@ -48,6 +48,7 @@
 #include <algorithm>
 
 #include "ee_internal.h"
+#include "ee_split3.cuh"
 #include "ee_umma.cuh"
 
 namespace ee {
@@ -76,24 +77,13 @@ struct UaSmem {
     static constexpr int bytes = at_bar + 64 + 1024;  // barriers, then alignment slack
 };
 
-// Eight floats as three 16-byte pieces of bf16 parts (each the rounding of
-// what the parts before it leave).
+// Eight floats as three 16-byte pieces of bf16 parts.
 __device__ __forceinline__ void ua_split8(const float (&x)[8], uint4 (&p)[3]) {
-    uint32_t w[3][4];
+    uint32_t w[4][3];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        float a = x[2 * e], b = x[2 * e + 1];
+    for (int e = 0; e < 4; ++e) split3(x[2 * e], x[2 * e + 1], w[e]);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);  // a in the low half
-            const uint32_t u = *reinterpret_cast<const uint32_t*>(&v);
-            w[k][e] = u;
-            a -= __uint_as_float(u << 16);
-            b -= __uint_as_float(u & 0xffff0000u);
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < 3; ++k) p[k] = make_uint4(w[k][0], w[k][1], w[k][2], w[k][3]);
+    for (int k = 0; k < 3; ++k) p[k] = make_uint4(w[0][k], w[1][k], w[2][k], w[3][k]);
 }
 __device__ __forceinline__ void ua_cp16(uint32_t dst, const void* src, int src_bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
