@@ -231,19 +231,6 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) {
         : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)));
     return d;
 }
-__device__ __forceinline__ float dot8s(const uint4 w, uint32_t xa) {
-    const float4 a = lds128f(xa);
-    const float4 b = lds128f(xa + 16);
-    float s = bflo(w.x) * a.x;
-    s = fmaf(bfhi(w.x), a.y, s);
-    s = fmaf(bflo(w.y), a.z, s);
-    s = fmaf(bfhi(w.y), a.w, s);
-    s = fmaf(bflo(w.z), b.x, s);
-    s = fmaf(bfhi(w.z), b.y, s);
-    s = fmaf(bflo(w.w), b.z, s);
-    s = fmaf(bfhi(w.w), b.w, s);
-    return s;
-}
 // Running dot products of one warp over ring stages: lane (c4, r8) = (lane /
 // 8, lane mod 8) holds the sums of rows r8, r8 + 8, r8 + 16 and r8 + 24 of
 // the tile over its own 16-byte column chunks, even and odd columns apart.
@@ -1511,8 +1498,7 @@ __global__ void __launch_bounds__(kSegThreads, 1) k_vocab_ring(VocabArgs v, int 
     s.full = reinterpret_cast<uint64_t*>(vr_smem + (size_t)stages * kSegChunk);
     s.empty = s.full + stages;
     float* xs = reinterpret_cast<float*>(s.empty + stages);
-    float* red = xs + ((v.d + 3) & ~3);              // [kRedSlots][kCW][32], then [kCW] norm partials
-    float* part = red + kRedSlots * kCW * 32 + kCW;  // [d / 8] partial dot products of one row
+    float* red = xs + ((v.d + 3) & ~3);  // [kRedSlots][kCW][32], then [kCW] norm partials
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         err_local = 0;
@@ -1561,17 +1547,45 @@ __global__ void __launch_bounds__(kSegThreads, 1) k_vocab_ring(VocabArgs v, int 
     if (nucleus) {
         nx = v.ctl->readout_token[0];
         if (nx < 0 || nx >= v.V) nx = 0;  // the readout pass flags an out-of-range token
-        const int Rc = v.d >> 3, tx = nx >> 5, lx_lane = nx & 31;
-        const uint4* W = reinterpret_cast<const uint4*>(v.U);
-        for (int c = threadIdx.x; c < Rc; c += kCT) {
-            const uint4 wv = __ldg(W + ((int64_t)tx * Rc + c) * 32 + lx_lane);
-            part[c] = dot8s(wv, saddr(xs + 8 * c));
+        // Summed as tile_gemv sums the row, bit for bit, so that equal rows tie:
+        // lane = the column chunks of one warp's column group there; the stages
+        // over the warps, whose sums warp 0 adds up in order.
+        constexpr int kGroup = kRedSlots * kCW / 2;  // stages whose sums fit red
+        float2* part = reinterpret_cast<float2*>(red);
+        const uint4* W = reinterpret_cast<const uint4*>(v.U) + ((int64_t)(nx >> 5) * (v.d >> 3)) * 32 + (nx & 31);
+        float2 acc = make_float2(0.f, 0.f);
+        for (int cb = 0; cb < nc; cb += kGroup) {
+            const int ce = min(nc, cb + kGroup);
+            for (int c = cb + w; c < ce; c += kCW) {
+                const int ccn = (int)(chunk_bytes(v.d, c) / 512);
+                float2 t = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int u = 0; u < kStageU; ++u) {
+                    const int ch = lane + u * kStageStep;
+                    if (ch >= ccn) continue;
+                    const uint4 wv = __ldg(W + (c * (kColsPerChunk / 8) + ch) * 32);
+                    const uint32_t xa = saddr(xs + c * kColsPerChunk + ch * 8);
+                    const float4 x0 = lds128f(xa), x1 = lds128f(xa + 16);
+                    t = fma2(make_float2(bflo(wv.x), bfhi(wv.x)), make_float2(x0.x, x0.y), t);
+                    t = fma2(make_float2(bflo(wv.y), bfhi(wv.y)), make_float2(x0.z, x0.w), t);
+                    t = fma2(make_float2(bflo(wv.z), bfhi(wv.z)), make_float2(x1.x, x1.y), t);
+                    t = fma2(make_float2(bflo(wv.w), bfhi(wv.w)), make_float2(x1.z, x1.w), t);
+                }
+                part[(c - cb) * 32 + lane] = t;
+            }
+            csync();
+            if (w == 0)
+                for (int c = cb; c < ce; ++c) acc = add2(acc, part[(c - cb) * 32 + lane]);
+            if (ce < nc) csync();
         }
-        csync();
-        if (threadIdx.x == 0) {
-            float acc = 0.f;
-            for (int c = 0; c < Rc; ++c) acc += part[c];
-            lx_s = acc;
+        if (w == 0) {
+            float sum = acc.x + acc.y;
+            sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+            sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+            float all = 0.f;
+#pragma unroll
+            for (int k = 0; k < kCW; ++k) all += __shfl_sync(0xffffffffu, sum, 4 * k);
+            if (lane == 0) lx_s = all;
         }
         csync();
         lx = lx_s;
@@ -1730,7 +1744,7 @@ __global__ void __launch_bounds__(kSegThreads, 1)
 
 bool vocab_ring_plan(int d, int n_sm, VocabRing& vr) {
     if (d % 8 || d <= 0 || n_sm <= 0) return false;
-    const size_t fixed = (size_t)(((d + 3) & ~3) + kRedSlots * kCW * 32 + kCW + d / 8) * 4 + 1024;
+    const size_t fixed = (size_t)(((d + 3) & ~3) + kRedSlots * kCW * 32 + kCW) * 4 + 1024;
     const size_t budget = 227 * 1024;
     if (fixed + 4 * (size_t)(kSegChunk + 16) > budget) return false;
     vr.G = n_sm;

@@ -90,6 +90,26 @@ def test_tiny_calibrate_matches_oracle(near_model, persistent, graphs):
         assert g["token"] == o["token"]
 
 
+@pytest.mark.parametrize("d", [256, 896, 2048])
+@pytest.mark.parametrize("persistent", [True, False])
+def test_equal_rows_tie_in_the_nucleus_mass(d, persistent):
+    """All rows of the unembedding equal: no token is more probable than the
+    readout's (token 0), whatever the logit rounds to, so the mass above it is
+    exactly 0: its own logit is summed in the order of the rows it is compared
+    with."""
+    from paper_2609_14144_gb300 import OPT_PERSISTENT, Engine
+
+    shape = TINY.replace(d_model=d, vocab=1000, n_layers=2, readout_layers=(1,))
+    model = synth.make_model(shape)
+    model["lm_head"] = np.repeat(model["lm_head"][:1], shape.vocab, axis=0)
+    eng = Engine(shape, model)
+    eng.set_option(OPT_PERSISTENT, int(persistent))
+    eng.prefill(synth.prompt(shape))
+    conf, member, mass = eng.calibrate(synth.calibration_stream(shape, 40), 0.9)
+    assert (mass == 0).all() and (member == 1).all(), mass
+    assert np.abs(conf - 1 / shape.vocab).max() <= 1e-8
+
+
 def test_tiny_calibrate_device_arrays_match_host(near_model):
     from paper_2609_14144_gb300 import DEVICE, Engine
 
