@@ -33,7 +33,8 @@
 //     the columns each): the high parts' after every chain of stages, added to
 //     running sums in registers, both after the last stage, when they write the
 //     split's partial sums part[s][row][n], which the consumer adds in split
-//     order as with the warp-level path.
+//     order as with the warp-level path.  (A small batch's chains have an
+//     accumulator each, all read after the last stage.)
 // The tensor core adds with truncation, so the error of a sum grows with the
 // number of steps it is carried through: with a whole K range in one chain a
 // 4099-position prompt was 2.0e-4 from 64 bits in its final state, with chains
@@ -419,11 +420,13 @@ int umma_splits(int64_t n_tiles, int K, int M, int n_sm) {
     return (int)std::max<int64_t>(1, want);
 }
 
-// Stages per chain.  A small batch: an accumulator for each.  A full block: 4,
-// fewer where a split of a 256-row batch (one CTA per SM)
-// would be shorter, so that short K ranges are summed no less exactly when
-// larger batches leave them fewer splits (feed-forward of 1000 rows at width 256:
-// error 3.4e-7 with chains of 4, 1.8e-7 in splits of one stage).
+// Stages per chain.  A small batch: as many as give every chain one of its four
+// accumulators (feed-forward of 33 rows against 64 bits, in chains of up to 24 and
+// now: 0.5B 1.2e-6, 4.1e-7; 1.5B 2.3e-6, 9.5e-7; 33 positions at 0.5B take 1227 us
+// for 1225).  A full block: 4, fewer where a split of a 256-row batch (one CTA per
+// SM) would be shorter, so that short K ranges are summed no less exactly when
+// larger batches leave them fewer splits (1000 rows at width 256: 3.4e-7 in
+// chains of 4, 1.9e-7 now, 1.8e-7 in splits of one stage).
 static int umma_chain(int64_t n_tiles, int K, int M, int S, int n_sm) {
     const int nk = (K + kUKStage - 1) / kUKStage;
     if (small_batch(M)) return ((nk + S - 1) / S + USmall::NA - 1) / USmall::NA;
