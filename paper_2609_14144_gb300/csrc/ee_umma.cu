@@ -431,7 +431,7 @@ static int umma_chain(int64_t n_tiles, int K, int M, int S, int n_sm) {
     const int nk = (K + kUKStage - 1) / kUKStage;
     if (small_batch(M)) return ((nk + S - 1) / S + USmall::NA - 1) / USmall::NA;
     const int64_t splits = std::max<int64_t>(1, n_sm / ((n_tiles + 3) / 4));
-    return (int)std::max<int64_t>(1, std::min<int64_t>(ULarge::CH, nk / splits));
+    return (int)std::max<int64_t>(1, std::min<int64_t>(ULarge::CH, (nk + splits - 1) / splits));
 }
 
 cudaError_t launch_mm_umma(const uint16_t* W, int64_t n_rows, int K, const uint16_t* x3, int ldx, int M, int S, int n_sm,

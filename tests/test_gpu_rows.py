@@ -212,6 +212,25 @@ def test_tcgen05_attention_row_and_key_edges(n, D, page):
                 assert rel_err(x, y) <= REL_TOL, t
 
 
+@pytest.mark.parametrize("n", [33, 65, 300, 700, 1000])
+@pytest.mark.parametrize("d", [256, 512, 1024, 1536])
+def test_products_in_chains_of_every_length(d, n):
+    """1280 inputs of the O projection: with 256, 512, 1024 and 1536 outputs a
+    full block's chains hold one, two, three and four stages, and the splits of
+    one, two, three and four blocks end in partial chains; a small batch's
+    chains have accumulators of their own.  Against one position at a time."""
+    shape = TINY.replace(d_model=d, n_heads=20, n_kv_heads=4, n_layers=2, readout_layers=(1,))
+    model = synth.make_model(shape)
+    prompt = synth.token_ids(shape.seed, 910 + n, n, shape.vocab)
+    a, b = (_engine(shape, model, n + 1, rows=r) for r in (1, 0))
+    a.prefill(prompt), b.prefill(prompt)
+    assert rel_err(a.hidden_final(), b.hidden_final()) <= PATH_TOL
+    assert rel_err(a.final_logits(), b.final_logits()) <= PATH_TOL
+    for t in sorted({0, n // 2, n - 2, n - 1}):  # layer 1's entries carry layer 0's products of that row
+        for x, y in zip(a.kv(1, t), b.kv(1, t)):
+            assert rel_err(x, y) <= REL_TOL, t
+
+
 @pytest.mark.parametrize("n", [48, 64, 400, 1000])
 def test_batched_products_round_like_short_chains(n):
     """The feed-forward of one layer (width 256: 8 and 22 stages of 32 columns
